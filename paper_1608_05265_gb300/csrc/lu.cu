@@ -5,8 +5,9 @@
 //
 // Right-looking, blocked by nb columns; each block is factored as panels of
 // at most 32 columns:
-//   panel    rows [j1, n) x the panel's columns, held in the shared memory
-//            of a cluster of up to 16 blocks for the whole factorisation
+//   panel    rows [j1, n) x the panel's columns, held by a cluster of up to
+//            16 blocks for the whole factorisation, in registers
+//            (lu_panel_reg_kernel) or beyond 16384 rows in shared memory
 //            (lu_panel_kernel): per column a block argmax, one exchange of
 //            candidates between the blocks (remote stores completing on the
 //            receivers' mbarriers), the pivot (first row of largest |a|)
@@ -18,8 +19,9 @@
 //   swap+U12 the other columns get that permutation (one gather per column:
 //            all sources read before any row is written), and right of the
 //            panel U12 = L11^-1 A12 is solved in shared memory
-//            (lu_swap_trsm_kernel); the block columns right of a panel are
-//            updated by the SIMT sgemm.
+//            (lu_swap_trsm32_kernel, lu_swap_trsm_kernel for wider blocks);
+//            the block columns right of a panel are updated by the SIMT
+//            sgemm.
 //   block    the block's exchanges, rebuilt as one permutation
 //            (lu_perm_kernel), reach every column outside the block, U12 of
 //            the block rows is solved, and the trailing matrix is updated by
@@ -31,7 +33,9 @@
 // memory), the off-diagonal parts by the library's sgemv or sgemm.  Every
 // sum is formed in a fixed order: runs are bit-identical.
 #include <cfloat>
+#include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -527,6 +531,372 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
   cl.sync();  // no block leaves while another may still read its published values
 }
 
+// One warp: right-looking forward substitution with the unit lower triangle
+// of a block of at most 32 rows on the 32 columns the lanes hold, u[i] the
+// value of row i: for each row p, u[i] -= L[i][p] u[p] for every i > p, so a
+// row's terms are added in the order of p and the steps of one p are
+// independent.  Lt is the triangle's transpose in shared memory, Lt[p][i];
+// rows of u past the block come out meaningless and are not used.
+__device__ __forceinline__ void warp_unit_lower_solve(const float (*Lt)[kLuPanelNb], float (&u)[kLuPanelNb]) {
+#pragma unroll
+  for (int p = 0; p < kLuPanelNb - 1; ++p)
+#pragma unroll
+    for (int g = p / 4; g < kLuPanelNb / 4; ++g) {
+      const float4 l = reinterpret_cast<const float4*>(Lt[p])[g];
+      if (4 * g + 0 > p) u[4 * g + 0] = fmaf(-l.x, u[p], u[4 * g + 0]);
+      if (4 * g + 1 > p) u[4 * g + 1] = fmaf(-l.y, u[p], u[4 * g + 1]);
+      if (4 * g + 2 > p) u[4 * g + 2] = fmaf(-l.z, u[p], u[4 * g + 2]);
+      if (4 * g + 3 > p) u[4 * g + 3] = fmaf(-l.w, u[p], u[4 * g + 3]);
+    }
+}
+
+// Four bytes into shared memory, asynchronously; src null: a zero (`any`: a
+// valid address, not read).
+__device__ __forceinline__ void lu_copy4(float* dst, const float* src, const float* any) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(lu_smem(dst)), "l"(src ? src : any),
+               "r"(src ? 4u : 0u) : "memory");
+}
+
+// Panel rows [j0, n) x columns [j0, j0 + nbp) (nbp <= 32) held in registers:
+// a thread owns RPT whole rows, block c of the cluster the panel rows
+// [c RPT T, (c + 1) RPT T) (T threads, rows tid + h T of the block's).  The
+// panel is a chain of nbp dependent pivot steps run by about one warp per
+// scheduler, so the latency and the number of a step's instructions bound
+// it, not arithmetic (32 FMA a row and step) or memory.  What keeps a step
+// short:
+//   no row moves.  A thread keeps its rows and, for each, a word position <<
+//   8 | block << 4 | warp; an exchange of rows q and p only renames two
+//   positions, and the row that became pivot row q is done.  The permutation
+//   falls out of the positions at the end;
+//   the update shifts.  x[j] holds column q + j, and x[j] = x[j + 1] - l
+//   u[j + 1] updates and renames in one instruction, so registers are
+//   indexed statically without unrolling the steps (two copies of the step,
+//   of 32 and 16 live columns).  Rows that are done run along, their values
+//   are not used any more, so nothing is predicated.  Multipliers go to
+//   shared memory (Ls, a column per step) and out at the end, a column at a
+//   time and coalesced;
+//   few warps.  Reading the pivot row costs 4 cycles of shared-memory return
+//   bandwidth per float4 and warp, whatever the broadcast (8 reads: 130
+//   cycles with 4 warps, 560 with 9), so rows per thread come before warps;
+//   two redux per level of the argmax (largest |a| as bits, then the smallest
+//   word, 24 cycles each): the word names the winner, so no ballot or
+//   shuffle follows;
+//   one barrier a step, and only the block's winning warp writes its row out
+//   and pushes it to every block of the cluster, its own included (st.async
+//   completing on the receiver's mbarrier); every thread waits on its own
+//   block's mbarrier only.  Every step has buffers and an mbarrier of its
+//   own, so nothing is re-armed, and the pivot rows are there at the end;
+//   the next column is updated first, so that its candidates are reduced
+//   while the other columns are updated.
+// A wait that runs out (2 s) sets *status; the thread then waits no more.
+// Candidates: |a| as bits, a NaN -1 (so that an all-NaN column keeps its
+// first row), no row -2; ties go to the smallest position.  A warp without a
+// row still offers its own word, so that every block always has a warp that
+// pushes.  ipiv and the permutation start as the identity, so that whatever a
+// wait that ran out leaves behind stays inside the panel.  The arithmetic of
+// every entry is that of lu_panel_kernel.
+// Measured at N 4608 (144 panels, launch list): 34 us a panel on average
+// against 120 of lu_panel_kernel, which held the rows in shared memory.
+constexpr int kRegPanelThreads = 256;  // at most; 65536 / 256 = 255 registers a thread
+constexpr size_t kRegPanelAlone = 196 * 1024;  // dynamic shared memory that keeps other kernels' blocks away
+template <int RPT, bool CLUSTER>
+__global__ void __launch_bounds__(kRegPanelThreads, 1)
+    lu_panel_reg_kernel(int n, float* __restrict__ A, int64_t lda, int j0, int nbp, int* __restrict__ ipiv,
+                        int* __restrict__ info, int* __restrict__ perm, int* __restrict__ status, int jp, int nbq,
+                        const int* __restrict__ perm_prev) {
+  constexpr int NB = kLuPanelNb;
+  constexpr int kMaxWarps = kRegPanelThreads / 32;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = CLUSTER ? (int)cl.num_blocks() : 1;
+  const int c = CLUSTER ? (int)cl.block_rank() : 0;
+  extern __shared__ __align__(16) float Ls[];  // multipliers: Ls[(q * RPT + h) * T + tid] (before that: L21 of the prologue)
+  __shared__ __align__(16) float row_s[NB];         // this block's candidate row, to push
+  __shared__ __align__(8) int2 wc[NB][kMaxWarps];   // each step's candidate (key, word) of each warp
+  __shared__ __align__(8) int2 rxc[NB][kLuPanelCluster];  // and of each block
+  __shared__ __align__(8) uint64_t bars[NB];
+  __shared__ __align__(16) float Ux[NB][NB + 4];  // prologue: U12 of this panel's columns
+  __shared__ __align__(16) float Lt[NB][NB];  // prologue: the previous block's L11, transposed
+  __shared__ int perm_s[3 * NB];
+  __shared__ int win[NB];                     // each step's pivot word
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = (int)blockDim.x;
+  const int R = n - j0;
+  float* const rx = Ls + NB * RPT * T;  // pivot row candidates: step q, block d at rx[(q * C + d) * NB]
+  float* G = A + j0 + (int64_t)j0 * lda;
+  auto live = [](int q) { return q < NB / 2 ? NB : NB / 2; };  // live columns of step q
+  for (int e = tid; e < NB * kMaxWarps; e += T) wc[e / kMaxWarps][e % kMaxWarps] = make_int2(-3, INT_MAX);
+  if (CLUSTER) {
+    for (int e = tid; e < NB * kLuPanelCluster; e += T) rxc[e / kLuPanelCluster][e % kLuPanelCluster] = make_int2(-3, INT_MAX);
+    if (tid < NB) {
+      lu_mbar_init(lu_smem(&bars[tid]));
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      lu_mbar_arm(lu_smem(&bars[tid]), (uint32_t)(C * (8 + 4 * live(tid))));
+    }
+  }
+  int pos[RPT];
+  const int row0 = c * RPT * T;
+#pragma unroll
+  for (int h = 0; h < RPT; ++h) pos[h] = row0 + h * T + tid;
+  float x[RPT][NB];
+  if (jp >= 0) {
+    // Prologue: the previous block [jp, j0) has not yet touched this panel's
+    // columns: rows that its exchanges replaced (at most NB) come from
+    // elsewhere, every block solves U12 = L11^-1 (the block's rows,
+    // exchanged), a warp with a column per lane, and its rows get
+    // A -= L21 U12.  Only original values of A are read here; U12 is written
+    // back at the end.  Every load is issued before the first is waited for:
+    // the triangle and U12's rows (first copy group), the rows themselves,
+    // L21 (second group).
+    int* const from = reinterpret_cast<int*>(rx);  // this block's rows' sources (RPT T <= NB NB ints)
+    const int nx = perm_prev[0];
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) from[h * T + tid] = pos[h];
+    for (int e = tid; e < 3 * NB; e += T) perm_s[e] = e < 3 * nbq ? perm_prev[1 + e] - j0 : 0;
+    for (int p = warp; p < nbq; p += T >> 5)
+      lu_copy4(&Lt[p][lane], lane < nbq ? A + (jp + lane) + (int64_t)(jp + p) * lda : nullptr, A);
+    __syncthreads();
+    if (tid < nx) {
+      const int to = perm_s[nbq + 2 * tid] - row0;
+      if (to >= 0 && to < RPT * T) from[to] = perm_s[nbq + 2 * tid + 1];
+    }
+    for (int p = warp; p < NB; p += T >> 5)
+      lu_copy4(&Ux[lane][p], lane < nbq && p < nbp ? G + perm_s[lane] + (int64_t)p * lda : nullptr, A);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+      const float* g = G + from[h * T + tid];
+      const bool in = pos[h] < R;
+#pragma unroll
+      for (int q = 0; q < NB; ++q, g += lda) x[h][q] = (q < nbp && in) ? *g : 0.f;
+    }
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+      const float* l = A + (j0 + (pos[h] < R ? pos[h] : 0)) + (int64_t)jp * lda;
+      float* to = Ls + h * T + tid;
+#pragma unroll 8
+      for (int q = 0; q < nbq; ++q, l += lda, to += RPT * T) lu_copy4(to, l, A);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+      float u[NB];
+#pragma unroll
+      for (int i = 0; i < NB; ++i) u[i] = Ux[i][lane];
+      warp_unit_lower_solve(Lt, u);
+#pragma unroll
+      for (int i = 0; i < NB; ++i) Ux[i][lane] = u[i];
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // (this thread's own copies)
+    __syncthreads();
+    const float* lq = Ls + tid;
+#pragma unroll 2
+    for (int q = 0; q < nbq; ++q, lq += RPT * T) {
+      float l[RPT];
+#pragma unroll
+      for (int h = 0; h < RPT; ++h) l[h] = lq[h * T];
+#pragma unroll
+      for (int g = 0; g < NB / 4; ++g) {
+        const float4 u4 = reinterpret_cast<const float4*>(Ux[q])[g];
+#pragma unroll
+        for (int h = 0; h < RPT; ++h) {
+          x[h][4 * g + 0] = fmaf(-l[h], u4.x, x[h][4 * g + 0]);
+          x[h][4 * g + 1] = fmaf(-l[h], u4.y, x[h][4 * g + 1]);
+          x[h][4 * g + 2] = fmaf(-l[h], u4.z, x[h][4 * g + 2]);
+          x[h][4 * g + 3] = fmaf(-l[h], u4.w, x[h][4 * g + 3]);
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+      const float* g = G + pos[h];
+      const bool in = pos[h] < R;
+#pragma unroll
+      for (int q = 0; q < NB; ++q, g += lda) x[h][q] = (q < nbp && in) ? *g : 0.f;
+    }
+  }
+  if (c == 0 && tid < nbp) {
+    ipiv[j0 + tid] = j0 + tid + 1;
+    perm[1 + tid] = j0 + tid;
+  }
+  // every block's mbarriers are initialised before any value is pushed; prologue reads done
+  if (CLUSTER) cl.sync();
+  else __syncthreads();
+  const int owner = c << 4 | warp;
+  int w[RPT];  // the rows' words; negative: no row
+#pragma unroll
+  for (int h = 0; h < RPT; ++h) w[h] = pos[h] < R ? pos[h] << 8 | owner : INT_MIN | owner;
+  // The thread's best row of column q, then the warp's best key and word.
+  int key, word, kh;
+  auto offer = [&](int q) {
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+      const uint32_t b = __float_as_uint(x[h][0]) & 0x7FFFFFFFu;
+      int k2 = b > 0x7F800000u ? -1 : (int)b;
+      if (w[h] < q << 8) k2 = -2;
+      if (h == 0) {
+        key = k2;
+        word = w[0];
+        kh = 0;
+      } else if (k2 > key || (k2 == key && w[h] < word)) {
+        key = k2;
+        word = w[h];
+        kh = h;
+      }
+    }
+    if (key < -1) word = 0x7FFFFF00 | owner;
+  };
+  auto first_best = [](int k2, int w2, int& top) -> int {
+    top = __reduce_max_sync(0xFFFFFFFFu, k2);
+    return __reduce_min_sync(0xFFFFFFFFu, k2 == top ? w2 : INT_MAX);
+  };
+  offer(0);
+  int top, best = first_best(key, word, top);
+  bool dead = false;
+  // One pivot step with W live columns (x[.][0 .. W-1]).
+  auto step = [&](auto width, int q) {
+    constexpr int W = decltype(width)::value;
+    if (lane == 0) wc[q][warp] = make_int2(top, best);
+    __syncthreads();
+    int2 cd = wc[q][lane % kMaxWarps];
+    int btop;
+    int bword = first_best(cd.x, cd.y, btop);
+    if ((bword & 15) == warp) {  // the block's candidate is this warp's
+      if (word == bword) {
+        float* to = CLUSTER ? row_s : rx + q * NB;
+#pragma unroll
+        for (int h = 0; h < RPT; ++h)
+          if (h == kh) {
+#pragma unroll
+            for (int g = 0; g < W / 4; ++g)
+              reinterpret_cast<float4*>(to)[g] = make_float4(x[h][4 * g], x[h][4 * g + 1], x[h][4 * g + 2], x[h][4 * g + 3]);
+          }
+      }
+      if (CLUSTER) {
+        __syncwarp();
+        // W / 4 lanes a destination: a float4 of the row each
+        constexpr int L = W / 4;
+        const int l = lane % L;
+        const float4 v = reinterpret_cast<const float4*>(row_s)[l];
+        const uint32_t slot = lu_smem(rx + (q * C + c) * NB + 4 * l), bar = lu_smem(&bars[q]);
+        if (lane < C) lu_push2(lu_mapa(lu_smem(&rxc[q][c]), lane), (uint32_t)btop, (uint32_t)bword, lu_mapa(bar, lane));
+#pragma unroll
+        for (int r = 0; r < kLuPanelCluster * L / 32; ++r) {
+          const int d = lane / L + r * (32 / L);
+          if (d < C) lu_push4(lu_mapa(slot, d), v, lu_mapa(bar, d));
+        }
+      }
+    }
+    const float* prow = rx + q * NB;
+    if (CLUSTER) {
+      if (!dead && !lu_mbar_try(lu_smem(&bars[q]), 0u) && !lu_mbar_wait(lu_smem(&bars[q]), 0u)) {
+        atomicCAS(status, 0, GBGEMM_ERR_DEVICE_TIMEOUT);
+        dead = true;
+      }
+      cd = rxc[q][lane % kLuPanelCluster];
+      bword = first_best(cd.x, cd.y, btop);
+      prow = rx + (q * C + min(bword >> 4 & 15, C - 1)) * NB;
+    } else {
+      __syncthreads();
+    }
+    float4 u[W / 4];
+#pragma unroll
+    for (int g = 0; g < W / 4; ++g) u[g] = reinterpret_cast<const float4*>(prow)[g];
+    const float d = u[0].x;
+    const float rcp = __frcp_rn(d);  // correctly rounded, as 1.0f / d
+    if (tid == 0) win[q] = bword;
+    // rows q and p trade places: p's row is done, q's row goes on at p
+#pragma unroll
+    for (int h = 0; h < RPT; ++h)
+      w[h] = w[h] == bword ? (q << 8 | owner) : (w[h] ^ owner) == q << 8 ? ((bword & ~255) | owner) : w[h];
+    float f[RPT];
+    if (fabsf(d) >= FLT_MIN) {  // 1 / d is finite
+#pragma unroll
+      for (int h = 0; h < RPT; ++h) f[h] = x[h][0] * rcp;
+    } else {  // a tiny pivot divides, a zero one scales nothing
+#pragma unroll
+      for (int h = 0; h < RPT; ++h) f[h] = d != 0.f ? x[h][0] / d : x[h][0];
+    }
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) Ls[(q * RPT + h) * T + tid] = f[h];
+    if (d != 0.f) {
+      // the next column first: its candidates are reduced while the rest is updated
+#pragma unroll
+      for (int h = 0; h < RPT; ++h) x[h][0] = fmaf(-f[h], u[0].y, x[h][1]);
+      offer(q + 1);
+      best = first_best(key, word, top);
+#pragma unroll
+      for (int j = 1; j < W - 1; ++j) {
+        const float4 u4 = u[(j + 1) / 4];
+        const float uj = (j + 1) % 4 == 0 ? u4.x : (j + 1) % 4 == 1 ? u4.y : (j + 1) % 4 == 2 ? u4.z : u4.w;
+#pragma unroll
+        for (int h = 0; h < RPT; ++h) x[h][j] = fmaf(-f[h], uj, x[h][j + 1]);
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < RPT; ++h)
+#pragma unroll
+        for (int j = 0; j < W - 1; ++j) x[h][j] = x[h][j + 1];
+      offer(q + 1);
+      best = first_best(key, word, top);
+    }
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) x[h][W - 1] = 0.f;
+  };
+  {
+    int q = 0;
+    for (; q < nbp && q < NB / 2; ++q) step(std::integral_constant<int, NB>{}, q);
+    for (; q < nbp; ++q) step(std::integral_constant<int, NB / 2>{}, q);
+  }
+  __syncthreads();
+  // Rows out at their final positions: multipliers a column at a time; the
+  // pivot rows and the prologue's U12 dealt over the blocks, a warp a row;
+  // ipiv and the first exactly zero pivot from block 0.
+#pragma unroll
+  for (int h = 0; h < RPT; ++h) {
+    pos[h] = w[h] >> 8;
+    const int qn = w[h] >= 0 && pos[h] < R ? min(pos[h], nbp) : 0;
+    float* g = G + pos[h];
+    const float* l = Ls + h * T + tid;
+#pragma unroll 8
+    for (int q = 0; q < NB; ++q, g += lda, l += RPT * T)
+      if (q < qn) *g = *l;
+  }
+  auto pivot_row = [&](int q) { return rx + (q * C + min(win[q] >> 4 & 15, C - 1)) * NB; };
+  for (int q = c + C * warp; q < nbp; q += C * (T >> 5))
+    if (q + lane < nbp) G[q + (int64_t)(q + lane) * lda] = pivot_row(q)[lane];
+  if (jp >= 0)
+    for (int k = c + C * warp; k < nbp; k += C * (T >> 5))
+      if (lane < nbq) A[(jp + lane) + (int64_t)(j0 + k) * lda] = Ux[lane][k];
+  if (c == 0 && warp == 0) {
+    const int p = lane < nbp ? win[lane] >> 8 : 0;
+    if (lane < nbp && p < R) ipiv[j0 + lane] = j0 + p + 1;  // (a wait that ran out may leave anything in p)
+    const unsigned zero = __ballot_sync(0xFFFFFFFFu, lane < nbp && *pivot_row(lane) == 0.f);
+    if (lane == 0 && zero && *info == 0) *info = j0 + __ffs(zero);
+  }
+  // The permutation: position s < nbp holds the row that came from src; a
+  // row of the first nbp that ended below them is an extra (no other row
+  // below moves: what an exchange sends down is always one of those rows,
+  // and all of them are the first rows of block 0's first warp).
+#pragma unroll
+  for (int h = 0; h < RPT; ++h) {
+    const int orig = row0 + h * T + tid;
+    if (orig < R && pos[h] < nbp) perm[1 + pos[h]] = j0 + orig;
+  }
+  if (c == 0 && warp == 0) {
+    const unsigned below = __ballot_sync(0xFFFFFFFFu, lane < nbp && pos[0] >= nbp && pos[0] < R);
+    if ((below >> lane) & 1u) {
+      const int x2 = __popc(below & ((1u << lane) - 1u));
+      perm[1 + nbp + 2 * x2] = j0 + pos[0];
+      perm[2 + nbp + 2 * x2] = j0 + lane;
+    }
+    if (lane == 0) perm[0] = __popc(below);
+  }
+  if (CLUSTER) cl.sync();  // no block leaves while another may still write to it
+}
+
 // Columns [c_lo, j0) and [j0 + nbp, c_hi): apply the row permutation of
 // pivot rows [j0, j0 + nbp) (all sources read before any row is written);
 // right of them, then U12 = L11^-1 A12, one thread per column, L11 and the
@@ -586,6 +956,69 @@ __global__ void __launch_bounds__(kSwapThreads) lu_swap_trsm_kernel(int n, float
     const int q = e % nbp, col = e / nbp;
     A[(j0 + q) + (int64_t)(c0 + col) * lda] = V[q * kXP + col];
   }
+}
+
+// The same for panels of at most 32 columns (any block of the default width
+// below n = 12288, and the panels inside wider blocks): a block of 128
+// threads takes 32 columns, so that n = 4608 gives every SM one, every load
+// of a thread (8 rows of the panel, 8 extras) is in flight at once, and one
+// warp solves U12 with a column per lane in registers.  Latency bounds it
+// (perm, then the gathers, then the solve): 7.5 us a launch on average at
+// N 4608 against 17.5 of the kernel above.
+constexpr int kNarrowCols = 32;
+constexpr int kNarrowThreads = 128;
+__global__ void __launch_bounds__(kNarrowThreads)
+    lu_swap_trsm32_kernel(float* __restrict__ A, int64_t lda, int j0, int nbp, const int* __restrict__ perm, int c_lo,
+                          int r_lo, int c_hi, int left_tiles) {
+  constexpr int NB = kLuPanelNb, NT = kNarrowThreads, PER = NB * kNarrowCols / NT;
+  __shared__ float V[kNarrowCols][NB + 1];
+  __shared__ __align__(16) float Lt[NB][NB];  // L11 transposed
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool left = (int)blockIdx.x < left_tiles;
+  const int c0 = left ? c_lo + (int)blockIdx.x * kNarrowCols : r_lo + ((int)blockIdx.x - left_tiles) * kNarrowCols;
+  const int ncol = min(c0 + kNarrowCols, left ? j0 : c_hi) - c0;
+  // lane = row of the panel or extra, warp + 4 v = column
+  const int next = perm[0];
+  const int src = lane < nbp ? perm[1 + lane] : 0;
+  const int xdst = lane < next ? perm[1 + nbp + 2 * lane] : 0;
+  const int xsrc = lane < next ? perm[2 + nbp + 2 * lane] : 0;
+  float* Ac = A + (int64_t)(c0 + warp) * lda;
+  float v[PER], w[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const bool col = warp + (NT / 32) * u < ncol;
+    v[u] = col && lane < nbp ? Ac[src + (int64_t)((NT / 32) * u) * lda] : 0.f;
+    w[u] = col && lane < next ? Ac[xsrc + (int64_t)((NT / 32) * u) * lda] : 0.f;
+  }
+  if (!left)
+#pragma unroll
+    for (int u = 0; u < NB / (NT / 32); ++u) {
+      const int p = warp + (NT / 32) * u;
+      Lt[p][lane] = lane < nbp && p < nbp ? A[(j0 + lane) + (int64_t)(j0 + p) * lda] : 0.f;
+    }
+  __syncthreads();  // every source is read before any row is written (the columns are this block's alone)
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+    if (warp + (NT / 32) * u < ncol && lane < next) Ac[xdst + (int64_t)((NT / 32) * u) * lda] = w[u];
+  if (!left) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) V[warp + (NT / 32) * u][lane] = v[u];
+    __syncthreads();
+    if (warp == 0) {
+      float x[NB];
+#pragma unroll
+      for (int i = 0; i < NB; ++i) x[i] = V[lane][i];
+      warp_unit_lower_solve(Lt, x);
+#pragma unroll
+      for (int i = 0; i < NB; ++i) V[lane][i] = x[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u) v[u] = V[warp + (NT / 32) * u][lane];
+  }
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+    if (warp + (NT / 32) * u < ncol && lane < nbp) Ac[(j0 + lane) + (int64_t)((NT / 32) * u) * lda] = v[u];
 }
 
 // The row exchanges of ipiv applied to one right-hand side per block, in
@@ -833,7 +1266,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   }
 }
 
-bool g_attr_done[64][7];
+bool g_attr_done[64][16];
 
 cudaError_t set_smem_once(const void* fn, int which, size_t bytes) {
   int dev = 0;
@@ -855,17 +1288,74 @@ int lu_panel_width(int rows) {
   return 1;
 }
 
+template <int RPT, bool CLUSTER>
+cudaError_t launch_panel_reg(int C, int T, int n, float* A, int64_t lda, int j0, int nbp, int* ipiv, int* info,
+                             int* perm, int* status, cudaStream_t s, int jp, int nbq, const int* perm_prev) {
+  const void* fn = (const void*)lu_panel_reg_kernel<RPT, CLUSTER>;
+  auto bytes = [](int blocks, int threads) {
+    return (size_t)kLuPanelNb * (RPT * threads + blocks * kLuPanelNb) * sizeof(float);
+  };
+  cudaError_t e = set_smem_once(fn, 6 + 2 * RPT + CLUSTER, std::max(bytes(CLUSTER ? kLuPanelCluster : 1, kRegPanelThreads), kRegPanelAlone));
+  if (e != cudaSuccess) return e;
+  static bool wide_set[64] = {};
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (CLUSTER && (dev < 0 || dev >= 64 || !wide_set[dev])) {
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) wide_set[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C, 1, 1);
+  cfg.blockDim = dim3(T, 1, 1);
+  // An SM of its own: beside a trailing update's blocks the steps take twice
+  // as long, so the launch asks for the shared memory such a block would need.
+  cfg.dynamicSmemBytes = std::max(bytes(C, T), kRegPanelAlone);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CLUSTER ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, lu_panel_reg_kernel<RPT, CLUSTER>, n, A, lda, j0, nbp, ipiv, info, perm, status, jp,
+                            nbq, perm_prev);
+}
+
 cudaError_t launch_lu_panel(int n, float* A, int64_t lda, int j0, int nbp, int* ipiv, int* info, int* perm,
                             int* status, cudaStream_t s, int jp, int nbq, const int* perm_prev) {
   if (jp >= 0 && (nbq <= 0 || nbq > kLuPanelNb || jp + nbq != j0 || !perm_prev)) return cudaErrorInvalidValue;
   if (nbp <= 0 || nbp > kLuPanelNb) return cudaErrorInvalidValue;
   const int R = n - j0;
+  // Rows in registers, up to 16384 of them: four warps a block (a warp per
+  // scheduler) with as many rows a thread as it takes, eight warps beyond 4.
+  // One block up to 384 rows (no exchange between blocks; a panel of 256
+  // rows 21 us, of 384 27.6, of 1024 45-49), else a cluster of 16 (a size
+  // the GPU allows by opt-in; 30 us up to 2048 rows, 35 up to 4096, 44 up to
+  // 6144) or, if that cannot be launched, of 8.
+  for (int C = R <= 384 ? 1 : kLuPanelCluster;;) {
+    const int per = (R + C - 1) / C;
+    const int rpt = per <= 128 ? 1 : per <= 256 ? 2 : per <= 384 ? 3 : 4;
+    const int T = ((per + rpt - 1) / rpt + 31) / 32 * 32;
+    if (T > kRegPanelThreads) break;
+    const int blocks = (R + rpt * T - 1) / (rpt * T);  // none without a row
+    auto launch = blocks > 1 ? (rpt == 1   ? launch_panel_reg<1, true>
+                                : rpt == 2 ? launch_panel_reg<2, true>
+                                : rpt == 3 ? launch_panel_reg<3, true>
+                                           : launch_panel_reg<4, true>)
+                             : (rpt == 1   ? launch_panel_reg<1, false>
+                                : rpt == 2 ? launch_panel_reg<2, false>
+                                : rpt == 3 ? launch_panel_reg<3, false>
+                                           : launch_panel_reg<4, false>);
+    cudaError_t e = launch(blocks, T, n, A, lda, j0, nbp, ipiv, info, perm, status, s, jp, nbq, perm_prev);
+    if (e == cudaSuccess || C != kLuPanelCluster) return e;
+    cudaGetLastError();
+    C = 8;
+  }
   const int pitch = lu_slab_pitch(nbp);
   const int cap = kLuPanelSlabBytes / (4 * pitch);  // slab rows a block holds
-  // one block up to 256 rows; 8 while a block's slab has at most 512 rows
-  // (a row per thread), else 16 (a cluster size the GPU allows by opt-in)
-  // (one block for more rows, two or three a thread, measured slower than the cluster's exchange)
-  int C = R <= 256 ? 1 : ((R + 7) / 8 <= kPanelThreads ? 8 : kLuPanelCluster);
+  int C = kLuPanelCluster;  // more rows than the registers of a cluster hold: in shared memory
   cudaError_t e = set_smem_once((const void*)lu_panel_kernel, 0, kLuPanelSlabBytes);
   if (e != cudaSuccess) return e;
   static bool wide_set[64] = {};
@@ -910,6 +1400,13 @@ cudaError_t launch_lu_swap_trsm(int n, float* A, int64_t lda, int j0, int nbp, c
   if (r_lo < 0) r_lo = j0 + nbp;
   if (nbp <= 0 || nbp > kLuMaxNb || c_lo < 0 || c_lo > j0 || r_lo < j0 + nbp || c_hi < r_lo || c_hi > n)
     return cudaErrorInvalidValue;
+  if (nbp <= kLuPanelNb) {
+    const int left_tiles = (j0 - c_lo + kNarrowCols - 1) / kNarrowCols;
+    const int tiles = left_tiles + (c_hi - r_lo + kNarrowCols - 1) / kNarrowCols;
+    if (tiles > 0)
+      lu_swap_trsm32_kernel<<<tiles, kNarrowThreads, 0, s>>>(A, lda, j0, nbp, perm, c_lo, r_lo, c_hi, left_tiles);
+    return cudaGetLastError();
+  }
   const int left_tiles = (j0 - c_lo + kTrsmCols - 1) / kTrsmCols;
   const int right_tiles = (c_hi - r_lo + kTrsmCols - 1) / kTrsmCols;
   if (left_tiles + right_tiles == 0) return cudaSuccess;
