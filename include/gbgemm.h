@@ -36,7 +36,16 @@
  *                           and six products are accumulated (hi*hi, hi*mid,
  *                           mid*hi, hi*lo3, mid*mid, lo3*hi).  Either way
  *                           the bound holds for every k.
- *   GBGEMM_PATH_AUTO        SPLIT_BF16 when k >= 128, else SIMT.
+ *   GBGEMM_PATH_AUTO        SPLIT_BF16 when k >= 128, else SIMT.  With the
+ *                           fixed heuristic (tuning mode 0, no pinned
+ *                           schedule) small outputs, short calls and long
+ *                           inner dimensions run the split without packed
+ *                           panels: the tiles' CTAs read and split the
+ *                           operands themselves, in one launch (two when k
+ *                           slices go through the workspace), with two
+ *                           accumulators per tile.  gbgemm_last_path and
+ *                           gbgemm_last_schedule report what the heuristic
+ *                           chose either way.
  *
  * Memory and streams.  All matrix pointers are DEVICE pointers owned by the
  * caller, who keeps them alive until the work queued on the handle's stream

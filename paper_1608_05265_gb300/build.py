@@ -20,9 +20,12 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libgbgemm.so")
 SOURCES = ["api.cu", "simt.cu", "split.cu", "noalloc.cu", "grouped.cu", "tuner.cu", "mlp.cu", "check.cu",
-           "gemv.cu", "lu.cu"]
+           "gemv.cu", "lu.cu", "direct.cu"]
+# Sources compiled once per set of macros (object name, source, macros).
+VARIANTS = [(f"direct_inst_p{p}_m{m}", "direct_inst.cu", [f"-DGBG_PARTS={p}", f"-DGBG_MODE_A={m}"])
+            for p in (2, 3) for m in (0, 1, 2)]
 HEADERS = [os.path.join(CSRC, h) for h in ("internal.h", "split_device.cuh", "simt_device.cuh", "gemm_kernel.cuh",
-                                            "grouped.h", "tuner.h", "mlp.h")] + \
+                                            "grouped.h", "tuner.h", "mlp.h", "direct.h", "direct_kernel.cuh")] + \
     [os.path.join(ROOT, "include", "gbgemm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
@@ -40,7 +43,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + [h for h in HEADERS if os.path.exists(h)] + \
+    deps = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(CSRC, v[1]) for v in VARIANTS] + [h for h in HEADERS if os.path.exists(h)] + \
         [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -51,9 +54,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT, exist_ok=True)
     cc = nvcc()
 
-    def compile_one(src: str) -> str:
-        obj = os.path.join(OUT, src.replace(".cu", ".o"))
-        cmd = [cc] + ARCH + FLAGS + ["-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(job) -> str:
+        name, src, macros = job
+        obj = os.path.join(OUT, name + ".o")
+        cmd = [cc] + ARCH + FLAGS + macros + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")
@@ -61,8 +65,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    jobs = VARIANTS + [(src[:-3], src, []) for src in SOURCES]  # the longest first
+    with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        objs = list(ex.map(compile_one, jobs))
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [cc] + ARCH + ["-shared", "-o", tmp] + objs
     r = subprocess.run(cmd, capture_output=True, text=True)

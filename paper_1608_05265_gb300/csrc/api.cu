@@ -317,15 +317,18 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
   }
   gbg::Problem p{ta, tb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
   gbg::Schedule d = default_schedule(h, h->path, m, n, k, batch);
+  bool fixed = true;  // the fixed heuristic chose
   const gbgemm_problem q1{transa, transb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
   if (batch == 1 && h->pinned_schedule >= 0 && schedule_allowed(h, q1, h->pinned_schedule)) {
     gbg::schedule_resolve(h->pinned_schedule, m, n, k, alpha, h->num_sms, &d);
+    fixed = false;
   } else if (h->tuning >= 1 && batch == 1) {
     const gbgemm_problem q{transa, transb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
     int best = -1;
     const int rc = choose_schedule(h, q, &best);
     if (rc != GBGEMM_OK) return rc;
     if (best >= 0) gbg::schedule_resolve(best, m, n, k, alpha, h->num_sms, &d);
+    fixed = best < 0;
   }
   const int path = d.path;
   const int simt_cfg = d.simt_cfg, split_bn = d.bn;
@@ -338,6 +341,24 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
     return GBGEMM_OK;
   }
   if (!split_supported(h)) return GBGEMM_ERR_UNSUPPORTED_DEVICE;
+  gbg::SplitCall c;
+  c.ta = ta; c.tb = tb; c.m = m; c.n = n; c.k = k; c.alpha = alpha; c.beta = beta;
+  c.A = A; c.lda = lda; c.B = B; c.ldb = ldb; c.C = C; c.ldc = ldc;
+  c.batch = batch; c.sa = sa; c.sb = sb; c.sc = sc;
+  c.status = h->d_status; c.num_sms = h->num_sms;
+  gbg::DirectPlan plan;
+  if (fixed && h->path == GBGEMM_PATH_AUTO && gbg::direct_plan(c, h->num_sms, &plan)) {
+    const int rc = ensure_workspace(h, gbg::direct_workspace_bytes(m, n, plan));
+    if (rc != GBGEMM_OK) return rc;
+    c.ws = h->ws;
+    if (prof_pair(h, &c.gemm_begin, &c.gemm_end) != cudaSuccess) return GBGEMM_ERR_CUDA;
+    if (gbg::launch_direct(c, plan, h->stream) != cudaSuccess) return GBGEMM_ERR_CUDA;
+    h->kernel_launches += plan.slices > 1 && !plan.in_cluster ? 2 : 1;
+    h->gemm_launches += 1;
+    h->last_path = GBGEMM_PATH_SPLIT_BF16;
+    h->last_schedule = gbg::schedule_encode_split(split_bn, d.raster, batch == 1 ? d.level : 0);
+    return GBGEMM_OK;
+  }
   // Workspace (one problem or a strided batch): control words, band counters
   // and row maxima (zeroed per call), the packed panels, and with split-K
   // (one problem, long k, too few tiles for the SMs) splitk x tiles raw
@@ -347,12 +368,8 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
   if (L.block > ((size_t)1 << 62) / (size_t)batch) return GBGEMM_ERR_ALLOC;
   int rc = ensure_workspace(h, L.total);
   if (rc != GBGEMM_OK) return rc;
-  gbg::SplitCall c;
-  c.ta = ta; c.tb = tb; c.m = m; c.n = n; c.k = k; c.alpha = alpha; c.beta = beta;
-  c.A = A; c.lda = lda; c.B = B; c.ldb = ldb; c.C = C; c.ldc = ldc;
-  c.batch = batch; c.sa = sa; c.sb = sb; c.sc = sc;
   c.bn = split_bn; c.raster = d.raster; c.splitk = splitk;
-  c.ws = h->ws; c.status = h->d_status; c.num_sms = h->num_sms;
+  c.ws = h->ws;
   h->kernel_launches += 1;  // the packing launch (the memset of the workspace head is not a kernel of ours)
   if (prof_pair(h, &c.gemm_begin, &c.gemm_end) != cudaSuccess) return GBGEMM_ERR_CUDA;
   if (gbg::launch_split_call(c, h->stream) != cudaSuccess) return GBGEMM_ERR_CUDA;

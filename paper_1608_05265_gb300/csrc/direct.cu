@@ -1,0 +1,172 @@
+// Host side of the direct split path (direct_kernel.cuh): which calls take it,
+// with which tiles and k slices, and the launch.
+#include <algorithm>
+#include <cmath>
+
+#include "direct.h"
+
+namespace gbg {
+namespace {
+
+int load_mode(bool kcontig, const float* x, int64_t ld, int64_t stride) {
+  if (!kcontig) return kRows;
+  return (ld & 3) == 0 && (stride & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 ? kVec : kScalar;
+}
+
+}  // namespace
+
+size_t direct_workspace_bytes(int64_t m, int64_t n, const DirectPlan& plan) {
+  if (plan.slices <= 1 || plan.in_cluster) return 0;
+  return (size_t)plan.slices * (size_t)((m + 127) / 128) * (size_t)((n + plan.bn - 1) / plan.bn) *
+         ((size_t)128 * plan.bn + kDirectExpInts) * 4;
+}
+
+namespace {
+
+// Estimated time (us) of a call on the packed path, as its launch chooses
+// tiles, pairs and k slices (split.cu, default_schedule): the launches, the
+// packing at its measured 4.8 TB/s, rounds of tiles at the measured time per
+// 32-deep chunk, the accumulators' way out, and the split-K reduction.
+// Against measurements at 256^3 .. 4096^3, ragged, tall, batched and long-k
+// shapes: within 15%.
+double packed_us(int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bool three) {
+  const double nkc = (double)panel_k_chunks(k);
+  const int64_t tm = (m + 127) / 128;
+  auto tiles = [&](int bn) { return (double)(tm * ((n + bn - 1) / bn) * batch); };
+  int bn = tiles(256) >= num_sms / 2 ? 256 : tiles(128) >= num_sms / 2 ? 128 : 64;
+  int s = batch == 1 ? choose_splitk((int64_t)tiles(256), k, num_sms) : 1;
+  if (s > 1) bn = 256;
+  double t = 12.5 + (three ? 10.0 : 8.0) * (double)k * (double)(m + n) * (double)batch / 4.8e6;
+  if (s > 1) t += 5.0;
+  const double chunks = std::ceil(nkc / s);
+  if (bn == 256 && tm >= 2 && (!three || nkc >= 8)) {
+    const double items = (double)((tm + 1) / 2 * ((n + 255) / 256) * batch) * s;
+    return t + std::ceil(items / (num_sms / 2)) * (chunks * (three ? 1.0 : 0.5) + 4.0);
+  }
+  const double per = bn == 256 ? 0.55 : bn == 128 ? 0.42 : 0.4;
+  return t + std::ceil(tiles(bn) * s / num_sms) * (chunks * per * (three ? 1.8 : 1.0) + 2.0);
+}
+
+// The same for a plan of the direct path.  Per 64-deep step 1.30 / 1.33 /
+// 1.58 us of a 64 / 128 / 256 wide tile (from 512 x 512 x 65536 without
+// slices), per 32-deep step with three parts 0.8 / 1.05; 1.2 times that with
+// operands whose rows are not 16-byte aligned.
+double direct_us(const DirectPlan& p, int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bool three,
+                 bool scalar) {
+  const int bm = p.pair ? 256 : 128;
+  const double ctas = (double)((m + bm - 1) / bm * ((n + p.bn - 1) / p.bn) * batch) * p.slices * (p.pair ? 2 : 1);
+  const double chunks = std::ceil((double)panel_k_chunks(k) / p.slices);
+  const double steps = three ? chunks : std::ceil(chunks / 2);
+  double step = three ? (p.bn == 64 ? 0.8 : 1.05) : p.bn == 64 ? 1.30 : p.bn == 128 ? 1.33 : 1.58;
+  if (scalar) step *= 1.2;
+  // Clusters do not fill the GPU's groups of SMs: of 152, clusters of 4, 8 and
+  // 16 CTAs reach 144, 120 and 112 (cudaOccupancyMaxActiveClusters).
+  const int size = (p.in_cluster ? p.slices : 1) * (p.pair ? 2 : 1);
+  double slots = num_sms * (size <= 2 ? 1.0 : size == 4 ? 144.0 / 152 : size == 8 ? 120.0 / 152 : 112.0 / 152);
+  if (three && ctas > slots) {  // two CTAs share an SM
+    slots *= 2;
+    step *= 2.2;
+  }
+  const double waves = std::ceil(ctas / slots);
+  const double out = p.bn * 0.03;  // a tile's way out: not hidden behind the next one
+  double t = (p.pair ? 9.0 : p.slices > 1 ? 6.5 : 4.5) + waves * (steps * step + out);
+  if (p.slices > 1 && p.pair) t += 2.5;
+  if (p.slices > 1 && !p.in_cluster) t += 4.0;
+  return t;
+}
+
+}  // namespace
+
+bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
+  const int64_t m = c.m, n = c.n, k = c.k, batch = c.batch;
+  if (c.lda >= (1 << 22) || c.ldb >= (1 << 22)) return false;  // offsets within a tile are 32 bits
+  const bool three = split_parts(k) == 2;
+  const int64_t nkc = panel_k_chunks(k);
+  const bool scalar = load_mode(c.ta == 1, c.A, c.lda, batch > 1 ? c.sa : 0) == kScalar ||
+                      load_mode(c.tb == 0, c.B, c.ldb, batch > 1 ? c.sb : 0) == kScalar;
+  // 8% in favour of the packed path: among 390 shapes drawn over the cases'
+  // ranges the direct path, where chosen, was 1.7 times as fast in the mean
+  // and at worst within 8% of it.
+  double best = 0.92 * packed_us(m, n, k, batch, num_sms, three);
+  bool found = false;
+  const size_t packed_bytes = split_layout(m, n, k, batch, 1, 256).total;
+  auto offer = [&](int bn, bool pair, int64_t slices, bool in_cluster) {
+    if (slices > 1) {  // steps of two chunks; no slice may be empty
+      const int64_t unit = three ? 1 : 2;
+      const int64_t per = ((nkc + slices - 1) / slices + unit - 1) / unit * unit;
+      const int64_t s = (nkc + per - 1) / per;
+      if (in_cluster ? s != slices || (nkc + slices - 1) / slices * (slices - 1) >= nkc : s < 2) return;
+      slices = s;
+      if ((nkc + slices - 1) / slices * (slices - 1) >= nkc) return;
+    }
+    DirectPlan p;
+    p.bn = bn; p.pair = pair; p.slices = (int)slices; p.in_cluster = in_cluster;
+    const int64_t bm = pair ? 256 : 128;
+    if ((m + bm - 1) / bm * ((n + bn - 1) / bn) * batch * slices > 0xFFFFFF) return;
+    // never more workspace than the packed path's, which callers may have reserved
+    if (direct_workspace_bytes(m, n, p) > packed_bytes) return;
+    const double t = direct_us(p, m, n, k, batch, num_sms, three, scalar);
+    if (t < best) {
+      best = t;
+      *plan = p;
+      found = true;
+    }
+  };
+  for (int s = 1; s <= 16; s *= 2) offer(64, false, s, true);
+  for (int s = 1; s <= 8; s *= 2) offer(128, true, s, true);
+  if (!three) {
+    offer(256, true, 1, true);
+    const int64_t tiles = (m + 255) / 256 * ((n + 255) / 256);
+    if (batch == 1 && tiles * 4 <= num_sms) offer(256, true, std::min<int64_t>(num_sms / (2 * tiles), 64), false);
+  }
+  return found;
+}
+
+cudaError_t launch_direct(const SplitCall& c, const DirectPlan& plan, cudaStream_t s) {
+  DirectArgs S{};
+  S.A = c.A; S.B = c.B; S.lda = c.lda; S.ldb = c.ldb; S.sa = c.sa; S.sb = c.sb;
+  S.m = c.m; S.n = c.n; S.k = c.k;
+  S.alpha = c.alpha; S.beta = c.beta;
+  S.C = c.C; S.ldc = c.ldc; S.sc = c.sc;
+  const int bm = plan.pair ? 256 : 128;
+  const int64_t tm = (c.m + bm - 1) / bm, tn = (c.n + plan.bn - 1) / plan.bn;
+  const int64_t items = tm * tn * c.batch * plan.slices;
+  if (items <= 0 || items > 0x3FFFFFFF) return cudaErrorInvalidValue;
+  S.tiles_m = (int)tm;
+  S.tiles_n = (int)tn;
+  S.nkc = (int)panel_k_chunks(c.k);
+  S.slices = plan.slices;
+  S.slice_chunks = (S.nkc + plan.slices - 1) / plan.slices;
+  if ((int64_t)(S.slices - 1) * S.slice_chunks >= S.nkc) return cudaErrorInvalidValue;  // no empty slice
+  S.cluster_slices = plan.in_cluster ? plan.slices : 1;
+  if (plan.in_cluster && plan.slices > 1 &&
+      (plan.bn % plan.slices || plan.slices * (plan.pair ? 2 : 1) > 16 || plan.bn > 128))
+    return cudaErrorInvalidValue;
+  S.partial = plan.slices > 1 && !plan.in_cluster ? static_cast<float*>(c.ws) : nullptr;
+  if (plan.slices > 1 && !plan.in_cluster && (c.batch != 1 || !c.ws)) return cudaErrorInvalidValue;
+  if (S.partial)
+    S.partial_exp = reinterpret_cast<int*>(S.partial + (size_t)plan.slices * ((c.m + 127) / 128) * tn * 128 * plan.bn);
+  S.status = c.status;
+  const int ma = load_mode(c.ta == 1, c.A, c.lda, c.batch > 1 ? c.sa : 0);
+  const int mb = load_mode(c.tb == 0, c.B, c.ldb, c.batch > 1 ? c.sb : 0);
+  const bool timed = c.gemm_begin && c.gemm_end;
+  cudaError_t e = timed ? cudaEventRecord(c.gemm_begin, s) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  auto launch = split_parts(c.k) == 2 ? (ma == kRows  ? launch_direct_mode<3, kRows>
+                                         : ma == kVec ? launch_direct_mode<3, kVec>
+                                                      : launch_direct_mode<3, kScalar>)
+                                      : (ma == kRows  ? launch_direct_mode<2, kRows>
+                                         : ma == kVec ? launch_direct_mode<2, kVec>
+                                                      : launch_direct_mode<2, kScalar>);
+  e = launch(plan, mb, S, items, s);
+  if (e == cudaSuccess && timed) e = cudaEventRecord(c.gemm_end, s);
+  if (e != cudaSuccess || !S.partial) return e;
+  SplitGemmArgs a;
+  a.m = c.m; a.n = c.n; a.k = c.k; a.alpha = c.alpha; a.beta = c.beta; a.C = c.C; a.ldc = c.ldc;
+  a.amaxA = nullptr; a.amaxB = nullptr; a.partial_exp = S.partial_exp;  // every slice has its own exponents
+  a.num_sms = c.num_sms; a.bn = plan.bn; a.splitk = plan.slices;
+  a.partial = S.partial;
+  return launch_splitk_reduce(a, s);
+}
+
+}  // namespace gbg

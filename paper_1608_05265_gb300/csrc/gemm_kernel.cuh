@@ -77,14 +77,6 @@ template <int STAGES, int MAXBN, bool PAIR = false>
 constexpr int gemm_smem_bytes() { return STAGES * (kBlockBytes + (PAIR ? MAXBN / 2 : MAXBN) * 128) + 1024 + 256; }
 constexpr int kGemmSmemBytes = gemm_smem_bytes<kStages, kMaxBN>();
 
-// The dependent launch of a kernel started with programmatic stream
-// serialisation may begin before this grid finishes; it waits (below) for
-// the grid's completion before it reads what the grid wrote.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// Wait until the grid this one depends on has completed and its memory is
-// visible (returns at once without such a dependency).
-__device__ __forceinline__ void wait_prerequisite_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Per-launch control words; zeroed before every launch together with the
 // band counters and the row maxima.
 struct WorkCtl {

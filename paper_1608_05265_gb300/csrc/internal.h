@@ -140,6 +140,24 @@ struct SplitCall {
 // reduction).
 cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s);
 
+// A split-path call without a packing pass (direct.cu): tiles of 128 x bn (bn
+// 64 or 128) or, pair, of 256 x bn (128 or 256), k in `slices` ranges, summed
+// in the cluster (bn a multiple of slices and at most 128, at most 16 CTAs) or
+// through c.ws (slices x the output's tiles raw 128 x bn accumulators).
+// Exponents of one slice's tile: whether any is set, those of its 128 rows and
+// (at most 256) columns.
+constexpr int kDirectExpInts = 1 + 128 + 256;
+struct DirectPlan {
+  int bn = 128;
+  bool pair = false;
+  int slices = 1;
+  bool in_cluster = true;
+};
+// Whether the direct path serves a call better than the packed one, and how.
+bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan);
+size_t direct_workspace_bytes(int64_t m, int64_t n, const DirectPlan& plan);
+cudaError_t launch_direct(const SplitCall& c, const DirectPlan& plan, cudaStream_t s);
+
 struct SplitGemmArgs {
   const uint32_t* amaxA; const uint32_t* amaxB;
   int64_t m, n, k;
@@ -149,6 +167,7 @@ struct SplitGemmArgs {
   int bn;
   int splitk = 1;
   float* partial = nullptr;
+  const int* partial_exp = nullptr;  // per slice and tile (kDirectExpInts ints) instead of amaxA, amaxB
 };
 
 // Number of k slices for a single split-path call with `tiles` output tiles

@@ -32,18 +32,49 @@
 namespace gbg {
 namespace {
 
+// The sum of the slices' accumulators of four rows and one column when some
+// slice's tile has exponents: every slice's are first brought to the largest
+// exponent of the row and of the column (a slice where either is zero
+// throughout has kNoExp there and adds nothing).
+__device__ __noinline__ float4 rescaled_sum(const float4* p, size_t slice_elems, int splitk, const int* pexp,
+                                            size_t pstride, int row, int col) {
+  constexpr int kNone = -(1 << 19);
+  float out[4];
+  for (int q = 0; q < 4; ++q) {
+    int er = 2 * kNone, ec = 2 * kNone;
+    for (int s = 0; s < splitk; ++s) {
+      er = max(er, pexp[s * pstride + 1 + row + q]);
+      ec = max(ec, pexp[s * pstride + 129 + col]);
+    }
+    float sum = 0.f;
+    for (int s = 0; s < splitk; ++s) {
+      const float acc = reinterpret_cast<const float*>(p + s * (slice_elems / 4))[q];
+      sum += scale_up(acc, pexp[s * pstride + 1 + row + q] - er + pexp[s * pstride + 129 + col] - ec);
+    }
+    out[q] = scale_up(sum, er + ec);
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
+}
+__device__ __forceinline__ void rescale_slices(float4& acc, const float4* p, size_t slice_elems, int splitk,
+                                               const int* pexp, size_t pstride, int row, int col) {
+  int any = 0;
+  for (int s = 0; s < splitk; ++s) any |= pexp[s * pstride];
+  if (any) acc = rescaled_sum(p, slice_elems, splitk, pexp, pstride, row, col);
+}
+
 // Split-K reduction: a thread per four consecutive rows i .. i+3 of one
 // column j of C (rows of a 128-row tile, so the partials are 16-byte
 // vectors), the slices' raw accumulators summed in slice order
 // (deterministic), then the epilogue of split_gemm_kernel: x 2^(e_i + f_j),
 // alpha, and beta C with one rounding of beta C and one fused multiply-add.
-// Every load of a thread is independent, so one pass over the grid keeps
+// With pexp the slices have exponents of their own (direct.cu).  Every load of a thread is independent, so one pass over the grid keeps
 // them all in flight.
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n, int bn, int tiles_m, int tiles_n,
                                                             int splitk, const float* __restrict__ partial,
                                                             const uint32_t* __restrict__ amaxA,
-                                                            const uint32_t* __restrict__ amaxB, float alpha,
-                                                            float beta, float* __restrict__ C, int64_t ldc) {
+                                                            const uint32_t* __restrict__ amaxB,
+                                                            const int* __restrict__ pexp, float alpha, float beta,
+                                                            float* __restrict__ C, int64_t ldc) {
   wait_prerequisite_grid();  // launched as a dependent of the GEMM
   const int64_t mq = (m + 3) / 4, total = mq * n;
   const size_t tile_elems = (size_t)128 * bn, slice_elems = (size_t)tiles_m * tiles_n * tile_elems;
@@ -64,7 +95,9 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
       for (int u = 0; u < 8; ++u)
         if (s0 + u < splitk) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
     }
-    const int fj = scale_exp_from_bits(amaxB[j]);
+    if (pexp) rescale_slices(acc, p, slice_elems, splitk, pexp + (tm * tiles_n + tn) * kDirectExpInts,
+                             (size_t)tiles_m * tiles_n * kDirectExpInts, (int)(i0 & 127), (int)(j - tn * bn));
+    const int fj = amaxB ? scale_exp_from_bits(amaxB[j]) : 0;
     float* c = C + i0 + j * ldc;
     const float a4[4] = {acc.x, acc.y, acc.z, acc.w};
     float o[4];
@@ -73,7 +106,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
       const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int e = scale_exp_from_bits(amaxA[i0 + q]) + fj;
+        const int e = amaxA ? scale_exp_from_bits(amaxA[i0 + q]) + fj : 0;
         const float v = (e >= -126 && e <= 127) ? a4[q] * __int_as_float((e + 127) << 23) : scalbnf(a4[q], e);
         o[q] = (beta != 0.f) ? fmaf(alpha, v, beta * c4[q]) : alpha * v;
       }
@@ -82,7 +115,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         if (i0 + q >= m) break;
-        const int e = scale_exp_from_bits(amaxA[i0 + q]) + fj;
+        const int e = amaxA ? scale_exp_from_bits(amaxA[i0 + q]) + fj : 0;
         const float v = (e >= -126 && e <= 127) ? a4[q] * __int_as_float((e + 127) << 23) : scalbnf(a4[q], e);
         c[q] = (beta != 0.f) ? fmaf(alpha, v, beta * c[q]) : alpha * v;
       }
@@ -283,7 +316,7 @@ cudaError_t launch_splitk_reduce(const SplitGemmArgs& a, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, splitk_reduce_kernel, a.m, a.n, a.bn, tm, tn, a.splitk, (const float*)a.partial,
-                            a.amaxA, a.amaxB, a.alpha, a.beta, a.C, a.ldc);
+                            a.amaxA, a.amaxB, a.partial_exp, a.alpha, a.beta, a.C, a.ldc);
 }
 
 }  // namespace gbg

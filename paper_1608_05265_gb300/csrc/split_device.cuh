@@ -38,6 +38,11 @@ __device__ __forceinline__ float scale_pow2(float x, int e) {
   return (x * 0x1p127f) * __int_as_float((s - 127 + 127) << 23);
 }
 
+// acc * 2^e: one multiply when 2^e is a normal float.
+__device__ __forceinline__ float scale_up(float acc, int e) {
+  return (e >= -126 && e <= 127) ? acc * __int_as_float((e + 127) << 23) : scalbnf(acc, e);
+}
+
 __device__ __forceinline__ void split_bf16(float xs, uint32_t& h, uint32_t& l) {
   const __nv_bfloat16 hb = __float2bfloat16_rn(xs);
   h = (uint32_t)__bfloat16_as_ushort(hb);
@@ -230,6 +235,14 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uin
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
+
+// The dependent launch of a kernel started with programmatic stream
+// serialisation may begin before this grid finishes; it waits (below) for
+// the grid's completion before it reads what the grid wrote.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Wait until the grid this one depends on has completed and its memory is
+// visible (returns at once without such a dependency).
+__device__ __forceinline__ void wait_prerequisite_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
