@@ -327,11 +327,13 @@ struct GroupedSched {
 };
 
 // Item (rr, cc) of a chunk in a packing CTA: row rr (0..127) of the band and
-// 8-wide k piece cc (0..3); item idx = tid + 256 * it, two per thread.
-// KCONTIG (element (r,p) at X[r*ld + p]): four consecutive items per row, so
-// a warp reads eight 128-byte row pieces.  !KCONTIG (X[r + p*ld]): 32
-// consecutive rows per warp and one piece per warp, so every load
-// instruction reads 128 contiguous bytes.
+// 8-wide k piece cc (0..3), two per thread.
+// KCONTIG (element (r,p) at X[r*ld + p]): item idx = tid + 256 * it, four
+// consecutive items per row, so a warp reads eight 128-byte row pieces and
+// its stores fill whole sectors.  !KCONTIG (X[r + p*ld]): 32 consecutive rows
+// per warp, so every load instruction reads 128 contiguous bytes, and two
+// neighbouring pieces of a row per thread, stored as whole 32-byte sectors
+// (store_split16).
 template <bool KCONTIG>
 __device__ __forceinline__ void item_of(int tid, int it, int& rr, int& cc) {
   const int idx = tid + 256 * it;
@@ -339,9 +341,9 @@ __device__ __forceinline__ void item_of(int tid, int it, int& rr, int& cc) {
     rr = idx >> 2;
     cc = idx & 3;
   } else {
-    const int w = idx >> 5;
-    cc = w & 3;
-    rr = (w >> 2) * 32 + (idx & 31);
+    const int w = tid >> 5;
+    cc = 2 * (w & 1) + it;
+    rr = (w >> 1) * 32 + (tid & 31);
   }
 }
 
@@ -401,11 +403,20 @@ __device__ __forceinline__ void pack_task_regs(const PackJob& P, uint32_t* smax)
       for (int it = 0; it < 2; ++it) {
         int rr, cc;
         item_of<KCONTIG>(tid, it, rr, cc);
+        const int mi = KCONTIG ? it : 0;  // !KCONTIG: both pieces are of one row
 #pragma unroll
-        for (int q = 0; q < 8; ++q) mxr[it] = max(mxr[it], __float_as_uint(x[c][it][q]) & 0x7FFFFFFFu);
-        if (r0 + rr < P.rows_alloc) {
+        for (int q = 0; q < 8; ++q) mxr[mi] = max(mxr[mi], __float_as_uint(x[c][it][q]) & 0x7FFFFFFFu);
+        if (KCONTIG && r0 + rr < P.rows_alloc) {
           if (blk2) store_split8_3(blk, blk2, (int)(kc & 1), rr, cc, x[c][it]);
           else store_split8(blk, rr, cc, x[c][it]);
+        }
+      }
+      if (!KCONTIG) {
+        int rr, cc;
+        item_of<KCONTIG>(tid, 0, rr, cc);
+        if (r0 + rr < P.rows_alloc) {
+          if (blk2) store_split16<true>(blk, blk2, (int)(kc & 1), rr, cc >> 1, x[c]);
+          else store_split16<false>(blk, nullptr, 0, rr, cc >> 1, x[c]);
         }
       }
     }

@@ -150,6 +150,54 @@ __device__ __forceinline__ void store_split8_3(uint8_t* blk, uint8_t* blk2, int 
   *reinterpret_cast<uint4*>(blk2 + rr * 128 + (((cc + 4 * half) ^ sw) << 4)) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
 
+// Splits of 8 values: hi and lo (mid), with three parts also lo3.
+template <bool THREE>
+__device__ __forceinline__ void split8(const float (&x)[8], uint32_t* h, uint32_t* l, uint32_t* t) {
+  const bool fin = all_finite8(x);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float a = x[2 * q], b = x[2 * q + 1];
+    h[q] = cvt_bf16x2(a, b);
+    const float r0 = a - bf16_lo(h[q]), r1 = b - bf16_hi(h[q]);
+    l[q] = cvt_bf16x2(r0, r1);
+    if (THREE) t[q] = cvt_bf16x2(r0 - bf16_lo(l[q]), r1 - bf16_hi(l[q]));
+    if (!fin) {  // Inf and NaN are all hi
+      const uint32_t keep = (isfinite(a) ? 0xFFFFu : 0u) | (isfinite(b) ? 0xFFFF0000u : 0u);
+      l[q] &= keep;
+      if (THREE) t[q] &= keep;
+    }
+  }
+}
+// 32 bytes in one store: whole L2 sectors.
+__device__ __forceinline__ void st_global32(uint8_t* p, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+// 16 consecutive k of row rr, the chunk's half kh: the two 16-byte pieces of
+// each part lie in one 32-byte sector, exchanged in odd rows.
+template <bool THREE>
+__device__ __forceinline__ void store_split16(uint8_t* blk, uint8_t* blk2, int half, int rr, int kh,
+                                              const float (&x)[2][8]) {
+  uint32_t h[2][4], l[2][4], t[2][4];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) split8<THREE>(x[c], h[c], l[c], t[c]);
+  const int sw = rr & 7;
+  const bool odd = sw & 1;
+  auto put = [&](uint8_t* row, int cc, const uint32_t (&w)[2][4]) {
+    uint32_t o[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      o[q] = odd ? w[1][q] : w[0][q];
+      o[4 + q] = odd ? w[0][q] : w[1][q];
+    }
+    st_global32(row + ((cc ^ (sw & 6)) << 4), o);
+  };
+  put(blk + rr * 128, 2 * kh, h);
+  put(blk + rr * 128, 2 * kh + 4, l);
+  if (THREE) put(blk2 + rr * 128, 2 * kh + 4 * half, t);
+}
+
 // ---------------------------------------------------------------------------
 // PTX wrappers (tcgen05, bulk copy, mbarrier)
 // ---------------------------------------------------------------------------
