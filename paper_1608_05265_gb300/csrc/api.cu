@@ -201,13 +201,23 @@ int gbgemm_reserve_workspace(gbgemm_handle* h, size_t bytes) {
 
 namespace {
 
+// SIMT tile.  Short k, where the tiles' ends cost more than their loads: 64 x
+// 64 up to half a million outputs (500 x 900 with k = 100: 12.5 us against
+// 14.4 and 20.7 of 128 x 64 and 128 x 128), beyond that 128 x 64 (2048 x
+// 1777, k = 64: 18.5 against 22.7; 4608^2, k = 32: 51 against 53).  Long k:
+// 64 x 64 for small outputs, else 128 x 128 (2048^3 TT: 448 against 473).
+int simt_config(int64_t m, int64_t n, int64_t k) {
+  if (k <= 128) return m * n <= ((int64_t)1 << 19) ? gbg::SIMT_64x64 : gbg::SIMT_128x64;
+  return m * n <= (int64_t)512 * 512 ? gbg::SIMT_64x64 : gbg::SIMT_128x128;
+}
+
 // The fixed heuristic's schedule of a call (tuning mode 0).  Path AUTO: split
 // from k = 128 on a GPU that has the split path, SIMT below.  Split: the
 // widest tile that still gives at least half of the SMs a tile (measured at
 // 2048^3: 128 BN-256 tiles beat 256 BN-128 tiles, 208 against 150 TFLOP/s),
 // tile rows in groups of 16, and for one problem with a long k and too few
-// tiles the k range cut into slices (keeping the widest tile).  SIMT: 64 x 64
-// for small outputs, else 128 x 128.
+// tiles the k range cut into slices (keeping the widest tile).  SIMT:
+// simt_config.
 gbg::Schedule default_schedule(const gbgemm_handle* h, int path, int64_t m, int64_t n, int64_t k, int64_t batch) {
   if (path == GBGEMM_PATH_AUTO) path = (k >= gbg::kSplitMinK && split_supported(h)) ? GBGEMM_PATH_SPLIT_BF16 : GBGEMM_PATH_SIMT;
   gbg::Schedule d{};
@@ -215,7 +225,7 @@ gbg::Schedule default_schedule(const gbgemm_handle* h, int path, int64_t m, int6
   d.raster = 16;
   d.level = 0;
   d.splitk = 1;
-  d.simt_cfg = (m * n <= (int64_t)512 * 512) ? gbg::SIMT_64x64 : gbg::SIMT_128x128;
+  d.simt_cfg = simt_config(m, n, k);
   auto tiles = [&](int64_t bm, int64_t bn) { return ((m + bm - 1) / bm) * ((n + bn - 1) / bn) * batch; };
   const int64_t half_sms = h->num_sms / 2;
   d.bn = tiles(128, 256) >= half_sms ? 256 : tiles(128, 128) >= half_sms ? 128 : 64;
@@ -531,8 +541,7 @@ int gbgemm_sgetrf(gbgemm_handle* h, int64_t n, float* A, int64_t lda, int* ipiv,
         const int64_t r = j1 + w, c = j1 + w;
         const gbg::Problem p{0, 0, rows, cols, w, -1.0f, 1.0f, A + r + j1 * lda, lda, A + j1 + c * lda, lda,
                              A + r + c * lda, lda};
-        const int cfg = rows * cols <= (int64_t)512 * 512 ? gbg::SIMT_64x64 : gbg::SIMT_128x128;
-        if (gbg::launch_simt(p, cfg, s) != cudaSuccess) return GBGEMM_ERR_CUDA;
+        if (gbg::launch_simt(p, simt_config(rows, cols, w), s) != cudaSuccess) return GBGEMM_ERR_CUDA;
         h->kernel_launches += 1;
       }
     }
