@@ -37,7 +37,21 @@
 //                   blocks of the result so that stores stay contiguous);
 //   warp 18         with beta != 0 and k <= 512, asks L2 for each tile's C
 //                   columns as soon as the tile is handed out, so that the
-//                   epilogue's reads of C find them there.
+//                   epilogue's reads of C find them there.  With staged jobs
+//                   (many problems) it also draws the tiles and leaves each
+//                   tile's job in shared memory, ahead of the producer.
+//
+// What bounds the many-problem instance is the two single-thread roles: at
+// 4096 problems up to 1024^3 the issuer spent about 80 cycles per MMA and the
+// producer about 330 per bulk copy against 32-128 cycles of tensor time per
+// MMA, and 1 KB copies or no stores at all changed the time by 3%.  Hence
+// tiles of up to 256 columns (half the MMAs and copies per result), edge
+// tiles that copy and multiply only the rows that exist, several chunks of a
+// small tile per ring slot, descriptors advanced by additions, and waits
+// whose first poll is inline: 1975 us for the packing and the GEMM became
+// 1709 us (4096^3: 317 -> 301 us, 8192^3: 2102 -> 2019 us by the last two
+// and by the epilogue's maxima being read before its wait).  Asking L2 for
+// the panels ahead of the copies did not help (2015 us).
 // Every wait is bounded: on expiry the kernel records GBGEMM_ERR_DEVICE_TIMEOUT,
 // raises a CTA-wide abort flag, drains its own copies and MMAs, frees TMEM
 // and returns.  Waiting threads sleep (mbarrier try_wait with a suspend
@@ -58,6 +72,7 @@ constexpr int kEpiWarps = 16;
 constexpr int kCpfWarp = 2 + kEpiWarps;            // the C prefetch warp
 constexpr int kGemmThreads = 32 * (kCpfWarp + 1);  // 19 warps, charged as 20: 96 registers per thread
 constexpr int kTileQ = 4;                          // tile-index queue between the roles
+constexpr int kAheadChunks = 6;                    // k chunks of tiles handed out ahead of the producer
 constexpr int kPackChunks = 4;                     // k chunks per packing task
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 // Suspend-time hint of the mbarrier waits: a waiting thread sleeps until the
@@ -74,7 +89,7 @@ constexpr uint64_t kDrainTimeoutNs = 4000000000ull;
 // most 128 columns the same memory holds a six-slot ring, and so it does for
 // pair tiles.
 template <int STAGES, int MAXBN, bool PAIR = false>
-constexpr int gemm_smem_bytes() { return STAGES * (kBlockBytes + (PAIR ? MAXBN / 2 : MAXBN) * 128) + 1024 + 256; }
+constexpr int gemm_smem_bytes() { return STAGES * (kBlockBytes + (PAIR ? MAXBN / 2 : MAXBN) * 128) + 1024 + 384; }
 constexpr int kGemmSmemBytes = gemm_smem_bytes<kStages, kMaxBN>();
 
 // Per-launch control words; zeroed before every launch together with the
@@ -86,7 +101,7 @@ struct WorkCtl {
 static_assert(sizeof(WorkCtl) == kSplitCtlBytes, "control block size");
 
 // Everything one tile needs.
-struct TileJob {
+struct alignas(16) TileJob {
   const uint8_t* a_src;     // A panel block of this tile row, k chunk 0
   const uint8_t* b_src;     // first B panel row of this tile column, k chunk 0
   size_t a_kstride;         // bytes between k chunks of the A panel
@@ -94,6 +109,8 @@ struct TileJob {
   int nkc;                  // k chunks
   int bn;                   // tile width: 64, 128 or 256
   int parts;                // 1: [hi | lo] panels, 3 products; 2: also compact lo3 panels, 6 products
+  int a_rows, b_rows;       // A and B panel rows copied per k chunk (b_rows: also the MMA's N; pairs: whole blocks)
+  int group;                // staged jobs: k chunks per ring slot (what fits beside each other), else 1
   int64_t a_part, b_part;   // byte offsets from the [hi | mid] panels to the compact lo3 panels
   int64_t m0, n0;           // tile origin in C
   int64_t m, n;             // problem extents
@@ -149,6 +166,7 @@ __device__ __forceinline__ void band_at(int pos, int ra, int rb, int gm, int nb0
 // z*as and its result at C + z*cs.  Band counters: problem z's A band a at
 // band_cnt[z*(ra+rb) + a], its B band b at band_cnt[z*(ra+rb) + ra + b].
 struct SingleSched {
+  static constexpr bool kStagedJobs = false;
   WorkCtl* ctl;
   int* band_cnt;
   const float* A; const float* B;
@@ -215,6 +233,7 @@ struct SingleSched {
     j.b_src = panel_rows(panelB + (size_t)z * ps, b_row0) + (size_t)kc0 * j.b_kstride;
     j.nkc = (nkc - kc0 < slice_chunks) ? nkc - kc0 : slice_chunks;
     j.bn = bn;
+    j.a_rows = 128; j.b_rows = bn; j.group = 1;
     j.partial = splitk > 1 ? partial + ((size_t)(sl * tiles_m + tm) * tiles_n + tn) * 128 * bn : nullptr;
     j.parts = parts; j.a_part = a_part; j.b_part = b_part;
     j.m0 = (int64_t)tm * 128; j.n0 = (int64_t)tn * bn;
@@ -254,19 +273,6 @@ struct SingleSched {
   }
 };
 
-// Device descriptor of one problem of a grouped batch on the split path.
-struct GroupDev {
-  const uint8_t* panelA; const uint8_t* panelB;
-  const uint32_t* amaxA; const uint32_t* amaxB;
-  float* C; int64_t ldc;
-  int64_t m, n;
-  int nkc, bn;
-  int64_t rowsA, rowsB;     // panel rows per k chunk
-  float alpha, beta;
-  int parts, pad_;
-  int64_t a_part, b_part;   // byte offsets to the compact lo3 panels (parts == 2)
-};
-
 // One 128-row band of one operand of a grouped problem, as the packers see it.
 struct PackBand {
   const float* X;
@@ -280,35 +286,21 @@ struct PackBand {
   int first_task, cnt;      // the band's first packing task and its counter
 };
 
-// Many problems: item t = (group, tile row, tile column), the items of one
-// problem together, problems in decreasing cost per tile, so that the cheap
-// tiles come last and fill the gaps.
+// Many problems: item t is one tile, its job written out by the host, the
+// tiles of one problem together, problems in decreasing cost per tile, so
+// that the cheap tiles come last and fill the gaps.  Edge tiles copy and
+// multiply only the panel rows that exist (op(B)'s rounded up to the MMA's
+// multiple of 16).
 struct GroupedSched {
+  static constexpr bool kStagedJobs = true;
   WorkCtl* ctl;
   int* band_cnt;
-  const int4* items;
-  const GroupDev* groups;
+  const TileJob* jobs;
   const PackBand* bands;
   const int* task_band;
   int n_items, n_tasks;
   __device__ __forceinline__ int num_items() const { return n_items; }
-  __device__ __forceinline__ TileJob job(int t) const {
-    const int4 it = items[t];
-    const GroupDev g = groups[it.x];
-    TileJob j;
-    j.a_src = g.panelA + (size_t)it.y * kBlockBytes;
-    j.b_src = panel_rows(g.panelB, (int64_t)it.z * g.bn);
-    j.a_kstride = (size_t)g.rowsA * 128;
-    j.b_kstride = (size_t)g.rowsB * 128;
-    j.nkc = g.nkc; j.bn = g.bn;
-    j.parts = g.parts; j.a_part = g.a_part; j.b_part = g.b_part;
-    j.m0 = (int64_t)it.y * 128; j.n0 = (int64_t)it.z * g.bn;
-    j.m = g.m; j.n = g.n;
-    j.amaxA = g.amaxA; j.amaxB = g.amaxB;
-    j.C = g.C; j.ldc = g.ldc; j.alpha = g.alpha; j.beta = g.beta;
-    j.partial = nullptr;
-    return j;
-  }
+  __device__ __forceinline__ TileJob job(int t) const { return jobs[t]; }
   __device__ __forceinline__ int num_pack_tasks() const { return n_tasks; }
   __device__ __forceinline__ PackJob pack_job(int i) const {
     const int b = task_band[i];
@@ -383,6 +375,14 @@ __device__ __forceinline__ void pack_task_regs(const PackJob& P, uint32_t* smax)
   const int nch = task_chunks(P);
   if (tid < 128) smax[tid] = 0u;
   uint32_t mxr[2] = {0u, 0u};
+  // The registers hold two chunks at a time: ask L2 for the task's other two
+  // now, so that their loads don't wait for memory (1731 -> 1709 us on 4096
+  // uneven problems up to 1024, where packing is half the time).
+  if (nch > 2) {
+    const int64_t r = r0 + (KCONTIG ? tid >> 1 : (tid & 3) * 32);
+    const int64_t p = (int64_t)(P.kc0 + 2) * 32 + (KCONTIG ? (tid & 1) * 32 : tid >> 2);
+    if (r < P.rows && p < P.k) prefetch_l2(KCONTIG ? P.X + r * P.ld + p : P.X + r + p * P.ld);
+  }
   for (int c0 = 0; c0 < nch; c0 += 2) {
     float x[2][2][8];
 #pragma unroll
@@ -495,7 +495,9 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
   const uint32_t drain_bar = bar0 + 8u * (2 * kStages + 4);
   auto tqf_bar = [&](int s) { return bar0 + 8u * (2 * kStages + 5 + s); };
   auto tqe_bar = [&](int s) { return bar0 + 8u * (2 * kStages + 5 + kTileQ + s); };
-  uint8_t* const tail = base_ptr + (bar0 - base) + 8 * (2 * kStages + 5 + 2 * kTileQ);
+  auto tqs_bar = [&](int s) { return bar0 + 8u * (2 * kStages + 5 + 2 * kTileQ + s); };
+  uint8_t* const tail = base_ptr + (bar0 - base) + 8 * (2 * kStages + 5 + 3 * kTileQ);
+  static_assert(8 * (2 * STAGES + 5 + 3 * kTileQ) + 16 + 4 * kTileQ <= 384, "barriers and tile queue");
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 4);
   volatile int* tile_q = reinterpret_cast<volatile int*>(tail + 16);          // kTileQ ints
@@ -510,6 +512,13 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
     if constexpr (PAIR) return S.job_pair(t, (int)crank);
     else return S.job(t);
   };
+  // Staged jobs: the scheduler warp leaves each tile's job in shared memory.
+  constexpr bool STAGED = Sched::kStagedJobs && !PAIR;
+  __shared__ TileJob job_q[STAGED ? kTileQ : 1];
+  auto take_job = [&](int slot, int t) -> TileJob {
+    if constexpr (STAGED) return job_q[slot];
+    else return job_of(t);
+  };
   auto wait_bar = [&](uint32_t bar, uint32_t parity) -> bool {
     return mbar_wait_hint(bar, parity, abort_flag, timeout_ns, kHintNs);
   };
@@ -519,7 +528,13 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), full_count); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), (PAIR ? 2 : 1) * kEpiWarps); }
     mbar_init(drain_bar, 1);
-    for (int s = 0; s < kTileQ; ++s) { mbar_init(tqf_bar(s), 1); mbar_init(tqe_bar(s), 2 + kEpiWarps); }
+    // a tile slot is read by the epilogue warps, the MMA issuer and one more:
+    // the producer where the scheduler warp fills it, else the prefetch warp
+    for (int s = 0; s < kTileQ; ++s) {
+      mbar_init(tqf_bar(s), 1);
+      mbar_init(tqe_bar(s), 2 + kEpiWarps);
+      mbar_init(tqs_bar(s), 1);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -573,33 +588,43 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       int tq = 0;
       uint32_t tqph = 0;
       int next_item = first_item;
-      int issued_phase[kStages];
-      bool issued[kStages];
-      for (int s = 0; s < kStages; ++s) { issued[s] = false; issued_phase[s] = 0; }
+      bool wrapped = false;  // every slot has been filled
       bool ok = true;
       while (ok) {
-        if (!mbar_wait_hint(tqe_bar(tq), tqph ^ 1u, abort_flag, timeout_ns, kHintNs)) {
+        if (!wait_bar(STAGED ? tqf_bar(tq) : tqe_bar(tq), STAGED ? tqph : tqph ^ 1u)) {
           raise_status(status, abort_flag);
           break;
         }
         int t;
-        if constexpr (PAIR) {
-          t = next_item;  // a fixed order, the same in both CTAs of the pair
-          next_item += num_pairs;
+        if constexpr (STAGED) {
+          t = tile_q[tq];
         } else {
-          t = atomicAdd(&S.ctl->tile_next, 1);
+          if constexpr (PAIR) {
+            t = next_item;  // a fixed order, the same in both CTAs of the pair
+            next_item += num_pairs;
+          } else {
+            t = atomicAdd(&S.ctl->tile_next, 1);
+          }
+          if (t >= num_items || *abort_flag) t = -1;
+          tile_q[tq] = t;
+          mbar_arrive(tqf_bar(tq));
         }
-        if (t >= num_items || *abort_flag) t = -1;
-        tile_q[tq] = t;
-        mbar_arrive(tqf_bar(tq));
-        if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
         if (t < 0) break;
-        const TileJob J = job_of(t);
-        const uint32_t b_bytes = (uint32_t)(PAIR ? J.bn / 2 : J.bn) * 128u;
-        // one ring slot per k chunk, and with three parts one more per pair
-        // of chunks (the compact [lo3 | lo3] block, loaded with the even chunk)
-        for (int kc = 0; kc < J.nkc && ok; ++kc) {
-          const int nparts = (J.parts == 2 && (kc & 1) == 0) ? 2 : 1;
+        const TileJob J = take_job(tq, t);
+        if constexpr (STAGED) {
+          mbar_arrive(tqs_bar(tq));
+          mbar_arrive(tqe_bar(tq));
+        }
+        if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
+        const uint32_t a_bytes = (uint32_t)J.a_rows * 128u;
+        const uint32_t b_bytes = (uint32_t)(PAIR ? J.b_rows / 2 : J.b_rows) * 128u;
+        // one ring slot per group of k chunks, and with three parts one more
+        // per pair of groups (the compact [lo3 | lo3] blocks, two chunks each,
+        // loaded with the even group)
+        const int grp = STAGED ? J.group : 1;
+        const bool even_only = J.parts == 2;
+        for (int kc = 0, gi = 0; kc < J.nkc && ok; kc += grp, ++gi) {
+          const int nparts = (even_only && (gi & 1) == 0) ? 2 : 1;
           for (int part = 0; part < nparts; ++part) {
             if (!wait_bar(empty_bar(stage), phase ^ 1u)) {
               raise_status(status, abort_flag);
@@ -610,19 +635,34 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
                                     : J.a_src + (size_t)kc * J.a_kstride;
             const uint8_t* b = part ? J.b_src + J.b_part + (size_t)(kc >> 1) * J.b_kstride
                                     : J.b_src + (size_t)kc * J.b_kstride;
-            mbar_arrive_expect_tx(full_bar(stage), A_BYTES + b_bytes);
-            bulk_copy_g2s(sA + stage * A_BYTES, a, A_BYTES, full_bar(stage));
-            bulk_copy_g2s(sB + stage * B_STAGE, b, b_bytes, full_bar(stage));
-            issued[stage] = true;
-            issued_phase[stage] = (int)phase;
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            const uint32_t bar = full_bar(stage), da = sA + stage * A_BYTES, db = sB + stage * B_STAGE;
+            if constexpr (STAGED) {
+              const int left = part ? ((J.nkc + 1) >> 1) - (kc >> 1) : J.nkc - kc;
+              const uint32_t cnt = (uint32_t)min(grp, left);
+              mbar_arrive_expect_tx(bar, cnt * (a_bytes + b_bytes));
+              // an operand of one row band has its chunks one after the other
+              if (J.a_kstride == a_bytes) bulk_copy_g2s(da, a, cnt * a_bytes, bar);
+              else
+                for (uint32_t c = 0; c < cnt; ++c) bulk_copy_g2s(da + c * a_bytes, a + c * J.a_kstride, a_bytes, bar);
+              if (J.b_kstride == b_bytes) bulk_copy_g2s(db, b, cnt * b_bytes, bar);
+              else
+                for (uint32_t c = 0; c < cnt; ++c) bulk_copy_g2s(db + c * b_bytes, b + c * J.b_kstride, b_bytes, bar);
+            } else {
+              mbar_arrive_expect_tx(bar, a_bytes + b_bytes);
+              bulk_copy_g2s(da, a, a_bytes, bar);
+              bulk_copy_g2s(db, b, b_bytes, bar);
+            }
+            if (++stage == kStages) { stage = 0; phase ^= 1u; wrapped = true; }
           }
         }
       }
-      // Let every copy this thread started land before the CTA can exit.
+      // Let every copy this thread started land before the CTA can exit: the
+      // slots before `stage` were last filled in this round of the ring, the
+      // others in the round before it.
       volatile int never = 0;
       for (int s = 0; s < kStages; ++s)
-        if (issued[s]) (void)mbar_wait(full_bar(s), (uint32_t)issued_phase[s], &never, kDrainTimeoutNs);
+        if (s < stage || wrapped)
+          (void)mbar_wait(full_bar(s), s < stage ? phase : phase ^ 1u, &never, kDrainTimeoutNs);
       // With pairs, rank 0's MMA commits release this CTA's slots by arriving
       // on its "empty" barriers: wait for the releases of the last fills, so
       // that no such arrival is still on its way when the CTA exits.
@@ -696,27 +736,31 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       int tq = 0;
       uint32_t tqph = 0;
       bool ok = true;
+      const uint64_t desc_a = make_desc_sw128(sA), desc_b = make_desc_sw128(sB);
       while (ok) {
         if (!mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs)) {
           raise_status(status, abort_flag);
           break;
         }
         const int t = tile_q[tq];
+        const TileJob J = t < 0 ? TileJob{} : take_job(tq, t);
         mbar_arrive(tqe_bar(tq));
         if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
         if (t < 0) break;
-        const TileJob J = job_of(t);
-        const uint32_t idesc = make_idesc_bf16(PAIR ? 256 : 128, J.bn);
+        const uint32_t idesc = make_idesc_bf16(PAIR ? 256 : 128, J.b_rows);
         if (!wait_bar(acce_bar(abuf), aphase ^ 1u)) {
           raise_status(status, abort_flag);
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(abuf * kMaxBN);
-        int s1 = 0;  // with three parts: the slot of the current [lo3 | lo3] block
-        for (int kc = 0; kc < J.nkc; ++kc) {
-          // the chunk's slot s0 holds [hi | lo] (or [hi | mid]); with three parts
-          // an even chunk also brings the pair's [lo3 | lo3] slot
+        int s1 = 0;  // with three parts: the slot of the current [lo3 | lo3] blocks
+        const int grp = STAGED ? J.group : 1;
+        const uint32_t a_step = (uint32_t)J.a_rows * 8u, b_step = (uint32_t)J.b_rows * 8u;  // a slot's next chunk, / 16 B
+        const bool three = PAIR ? THREE : J.parts == 2;
+        for (int kc0 = 0, gi = 0; kc0 < J.nkc; kc0 += grp, ++gi) {
+          // the group's slot s0 holds [hi | lo] (or [hi | mid]) per chunk; with
+          // three parts an even group also brings the pair's [lo3 | lo3] slot
           const int s0 = stage;
           const uint32_t ph0 = phase;
           if (!wait_bar(full_bar(s0), ph0)) {
@@ -724,60 +768,60 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
             ok = false;
             break;
           }
-          if (J.parts == 2 && (kc & 1) == 0) {
+          if (three && (gi & 1) == 0) {
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
             s1 = stage;
-            if (!mbar_wait_hint(full_bar(s1), phase, abort_flag, timeout_ns, kHintNs)) {
+            if (!wait_bar(full_bar(s1), phase)) {
               raise_status(status, abort_flag);
               ok = false;
               break;
             }
           }
           tc_fence_after();
-          const uint32_t a_addr = sA + s0 * A_BYTES;
-          const uint32_t b_addr = sB + s0 * B_STAGE;
-          const uint32_t a3_addr = sA + s1 * A_BYTES + 64u * (uint32_t)(kc & 1);
-          const uint32_t b3_addr = sB + s1 * B_STAGE + 64u * (uint32_t)(kc & 1);
+          auto mma = [&](uint64_t x, uint64_t y, uint32_t acc) {
+            if constexpr (PAIR) mma_bf16_pair(d_tmem, x, y, idesc, acc);
+            else mma_bf16(d_tmem, x, y, idesc, acc);
+          };
+          // descriptors: start addresses count 16-byte units, so the second
+          // half of a chunk is 2 and its [lo | mid] columns 4 units on
+          uint64_t da = desc_a + (uint64_t)(s0 * (A_BYTES / 16)), db = desc_b + (uint64_t)(s0 * (B_STAGE / 16));
+          const int kend = STAGED ? min(kc0 + grp, J.nkc) : kc0 + 1;
+          for (int kc = kc0; kc < kend; ++kc) {
+            const uint32_t acc0 = kc > 0 ? 1u : 0u;
+            if (three) {
+              // [hi | mid] and the pair's [lo3 | lo3]: hi*hi, hi*mid, mid*hi, hi*lo3, mid*mid, lo3*hi
+              const uint32_t pj = STAGED ? (uint32_t)((kc - (gi & ~1) * grp) >> 1) : 0u;  // its block in slot s1
+              const uint32_t at3 = 4u * (uint32_t)(kc & 1);
+              const uint64_t a3 = desc_a + (uint64_t)(s1 * (A_BYTES / 16) + pj * a_step + at3);
+              const uint64_t b3 = desc_b + (uint64_t)(s1 * (B_STAGE / 16) + pj * b_step + at3);
 #pragma unroll
-          for (int kk = 0; kk < 2; ++kk) {
-            const uint64_t ah = make_desc_sw128(a_addr + 32u * kk);
-            const uint64_t al = make_desc_sw128(a_addr + 64u + 32u * kk);
-            const uint64_t bh = make_desc_sw128(b_addr + 32u * kk);
-            const uint64_t bl = make_desc_sw128(b_addr + 64u + 32u * kk);
-            if constexpr (PAIR) {
-              mma_bf16_pair(d_tmem, ah, bh, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-              mma_bf16_pair(d_tmem, ah, bl, idesc, 1u);
-              mma_bf16_pair(d_tmem, al, bh, idesc, 1u);
-              if constexpr (THREE) {
-                // with three parts: hi*lo3 + mid*mid + lo3*hi (al, bl above are mid)
-                const uint64_t a3 = make_desc_sw128(a3_addr + 32u * kk);
-                const uint64_t b3 = make_desc_sw128(b3_addr + 32u * kk);
-                mma_bf16_pair(d_tmem, ah, b3, idesc, 1u);
-                mma_bf16_pair(d_tmem, al, bl, idesc, 1u);
-                mma_bf16_pair(d_tmem, a3, bh, idesc, 1u);
+              for (int kk = 0; kk < 2; ++kk) {
+                mma(da + 2 * kk, db + 2 * kk, kk > 0 ? 1u : acc0);
+                mma(da + 2 * kk, db + 2 * kk + 4, 1u);
+                mma(da + 2 * kk + 4, db + 2 * kk, 1u);
+                mma(da + 2 * kk, b3 + 2 * kk, 1u);
+                mma(da + 2 * kk + 4, db + 2 * kk + 4, 1u);
+                mma(a3 + 2 * kk, db + 2 * kk, 1u);
               }
             } else {
-              mma_bf16(d_tmem, ah, bh, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-              mma_bf16(d_tmem, ah, bl, idesc, 1u);
-              mma_bf16(d_tmem, al, bh, idesc, 1u);
-              if (J.parts == 2) {
-                // with three parts: hi*lo3 + mid*mid + lo3*hi (al, bl above are mid)
-                const uint64_t a3 = make_desc_sw128(a3_addr + 32u * kk);
-                const uint64_t b3 = make_desc_sw128(b3_addr + 32u * kk);
-                mma_bf16(d_tmem, ah, b3, idesc, 1u);
-                mma_bf16(d_tmem, al, bl, idesc, 1u);
-                mma_bf16(d_tmem, a3, bh, idesc, 1u);
+#pragma unroll
+              for (int kk = 0; kk < 2; ++kk) {
+                mma(da + 2 * kk, db + 2 * kk, kk > 0 ? 1u : acc0);
+                mma(da + 2 * kk, db + 2 * kk + 4, 1u);
+                mma(da + 2 * kk + 4, db + 2 * kk, 1u);
               }
             }
+            da += a_step;
+            db += b_step;
           }
+          // frees the slots (with pairs in both CTAs) once these MMAs have read them
+          const bool free3 = three && ((gi & 1) == 1 || kc0 + grp >= J.nkc);
           if constexpr (PAIR) {
-            mma_commit_pair(empty_bar(s0), 0x3);  // frees the slot in both CTAs once these MMAs have read it
-            if constexpr (THREE) {
-              if ((kc & 1) == 1 || kc == J.nkc - 1) mma_commit_pair(empty_bar(s1), 0x3);
-            }
+            mma_commit_pair(empty_bar(s0), 0x3);
+            if (free3) mma_commit_pair(empty_bar(s1), 0x3);
           } else {
-            mma_commit(empty_bar(s0));  // frees the slot once these MMAs have read it
-            if (J.parts == 2 && ((kc & 1) == 1 || kc == J.nkc - 1)) mma_commit(empty_bar(s1));
+            mma_commit(empty_bar(s0));
+            if (free3) mma_commit(empty_bar(s1));
           }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -808,18 +852,35 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
         ok = mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs) ? 1 : 0;
         if (ok) {
           t = tile_q[tq];
-          mbar_arrive(tqe_bar(tq));
+          if (!STAGED) mbar_arrive(tqe_bar(tq));
         }
       }
       ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
       t = __shfl_sync(0xFFFFFFFFu, t, 0);
-      if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
       if (!ok) {
         if (lane == 0) raise_status(status, abort_flag);
         break;
       }
       if (t < 0) break;
-      const TileJob J = job_of(t);
+      if constexpr (STAGED) __syncwarp();  // lane 0 has seen the job complete
+      const TileJob J = take_job(tq, t);
+      if constexpr (STAGED) {
+        __syncwarp();  // every lane has read it
+        if (lane == 0) mbar_arrive(tqe_bar(tq));
+      }
+      if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
+      // maxima were built by the packing: read them through L2, before the
+      // wait, like the first columns' below
+      const int64_t i = J.m0 + q * 32 + lane;
+      const bool row_ok = i < J.m;
+      const int cols = (J.bn / (kEpiWarps / 4)) > 32 ? J.bn / (kEpiWarps / 4) : 32;
+      const int c_begin = part * cols, c_end = (c_begin + cols < J.bn) ? c_begin + cols : J.bn;
+      auto col_bits = [&](int c0) -> uint32_t {
+        const int64_t jl = J.n0 + c0 + lane;
+        return (c0 < c_end && jl < J.n) ? __ldcg(J.amaxB + jl) : 0u;
+      };
+      const uint32_t ea_bits = row_ok ? __ldcg(J.amaxA + i) : 0u;
+      uint32_t eb_bits = col_bits(c_begin);
       if (lane == 0) ok = wait_bar(accf_bar(abuf), aphase) ? 1 : 0;
       ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
       if (!ok) {
@@ -827,15 +888,10 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
         break;
       }
       tc_fence_after();
-      const int64_t i = J.m0 + q * 32 + lane;
-      const bool row_ok = i < J.m;
-      // maxima were built by other CTAs' atomics: read them through L2
-      const int ea = row_ok ? scale_exp_from_bits(__ldcg(J.amaxA + i)) : 0;
+      const int ea = scale_exp_from_bits(ea_bits);
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(abuf * kMaxBN);
       float* const crow = J.C + i;
       constexpr int EC = 32;
-      const int cols = (J.bn / (kEpiWarps / 4)) > 32 ? J.bn / (kEpiWarps / 4) : 32;
-      const int c_begin = part * cols, c_end = (c_begin + cols < J.bn) ? c_begin + cols : J.bn;
       if (J.partial && J.m0 < J.m) {
         // split-K slice: the raw accumulator, whole tile, 32 consecutive rows
         // per warp store (not for the empty odd half of a last pair, which
@@ -859,8 +915,8 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
 #pragma unroll
           for (int jj = 0; jj < EC; ++jj) cv[jj] = (row_ok && jj < jmax) ? __ldcs(cp + jj * J.ldc) : 0.f;
         }
-        const int64_t jl = J.n0 + c0 + lane;
-        const int eb_l = (lane < EC && jl < J.n) ? scale_exp_from_bits(__ldcg(J.amaxB + jl)) : 0;
+        const int eb_l = scale_exp_from_bits(eb_bits);
+        eb_bits = col_bits(c0 + EC);
         uint32_t r[EC];
         tmem_ld32(taddr + (uint32_t)c0, r);
         if (__all_sync(0xFFFFFFFFu, ea == 0 && eb_l == 0)) {
@@ -906,25 +962,66 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       if (++abuf == 2) { abuf = 0; aphase ^= 1u; }
     }
   } else if (warp == kCpfWarp) {
-    // ---------------- C prefetch ----------------
+    // ---------------- C prefetch; staged jobs: also the tile scheduler ----------------
     // With beta != 0 the epilogue reads the tile's C: ask L2 for it as soon
     // as the tile is handed out, one to three tiles ahead of the epilogue.
+    // With staged jobs this warp draws the tiles: the counter and the job are
+    // two dependent trips to L2 or memory, which the producer and the MMA
+    // issuer each waited for at every tile.  It stays ahead of the producer
+    // by one tile, or by up to three while those hold fewer than kAheadChunks
+    // k chunks together, so that a CTA never sits on work others could do.
     int tq = 0;
     uint32_t tqph = 0;
+    int sq = 0, ahead = 0, ahead_chunks = 0;  // lane 0, staged: tiles the producer has not begun
+    uint32_t sqph = 0;
     for (;;) {
       int ok = 1, t = -1;
-      if (lane == 0) {
-        ok = mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs) ? 1 : 0;
-        if (ok) {
-          t = tile_q[tq];
-          mbar_arrive(tqe_bar(tq));
+      if constexpr (STAGED) {
+        if (lane == 0) {
+          while (ok && ahead > 0 && (ahead_chunks >= kAheadChunks || ahead == kTileQ - 1)) {
+            ok = wait_bar(tqs_bar(sq), sqph) ? 1 : 0;
+            --ahead;
+            ahead_chunks -= job_q[sq].nkc;
+            if (++sq == kTileQ) { sq = 0; sqph ^= 1u; }
+          }
+          ok = ok && wait_bar(tqe_bar(tq), tqph ^ 1u) ? 1 : 0;
+          if (ok) {
+            t = atomicAdd(&S.ctl->tile_next, 1);
+            if (t >= num_items || *abort_flag) t = -1;
+          } else {
+            raise_status(status, abort_flag);
+          }
         }
+        ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+        t = __shfl_sync(0xFFFFFFFFu, t, 0);
+        if (!ok) break;
+        constexpr int JW = sizeof(TileJob) / 16;
+        static_assert(sizeof(TileJob) % 16 == 0 && JW <= 32, "one 16-byte piece per lane");
+        __syncwarp();  // lane 0 has seen the slot free
+        if (t >= 0 && lane < JW)
+          reinterpret_cast<uint4*>(&job_q[tq])[lane] = __ldg(reinterpret_cast<const uint4*>(S.jobs + t) + lane);
+        __syncwarp();
+        if (lane == 0) {
+          tile_q[tq] = t;
+          mbar_arrive(tqf_bar(tq));
+        }
+        if (t < 0) break;
+        ++ahead;
+        ahead_chunks += job_q[tq].nkc;
+      } else {
+        if (lane == 0) {
+          ok = mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs) ? 1 : 0;
+          if (ok) {
+            t = tile_q[tq];
+            mbar_arrive(tqe_bar(tq));
+          }
+        }
+        ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+        t = __shfl_sync(0xFFFFFFFFu, t, 0);
+        if (!ok || t < 0) break;
       }
-      ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-      t = __shfl_sync(0xFFFFFFFFu, t, 0);
+      const TileJob J = take_job(tq, t);
       if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
-      if (!ok || t < 0) break;
-      const TileJob J = job_of(t);
       // Only short tiles (k <= 512), whose epilogue rather than their MMAs
       // sets the pace, are prefetched: for long ones the C reads overlap the
       // next tile's MMAs anyway, and prefetching several 128 KB tiles ahead

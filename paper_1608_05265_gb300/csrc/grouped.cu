@@ -101,7 +101,11 @@ bool config_legal(const gbgemm_problem& q, int cfg) {
 }
 
 int default_config(const gbgemm_problem& q) {
-  if (q.k >= kSplitShortK && q.alpha != 0.0f) return q.n <= 64 ? GBGEMM_CFG_SPLIT_BN64 : GBGEMM_CFG_SPLIT_BN128;
+  // Edge tiles cost what they hold, so the widest tile that n fills: on 4096
+  // problems up to 1024 a plan took 1744 us with 256 columns from n = 129 on,
+  // 1778 from 193, 1810 from 257 and 1975 never; up to 256, 355 against 364.
+  if (q.k >= kSplitShortK && q.alpha != 0.0f)
+    return q.n <= 64 ? GBGEMM_CFG_SPLIT_BN64 : q.n <= 128 ? GBGEMM_CFG_SPLIT_BN128 : GBGEMM_CFG_SPLIT_BN256;
   // SIMT: the tile shape with the least padded area (ties to the larger tile)
   auto area = [&](int64_t bm, int64_t bn) { return ((q.m + bm - 1) / bm) * bm * (((q.n + bn - 1) / bn) * bn); };
   const int64_t a_big = area(128, 128), a_wide = area(128, 64), a_small = area(64, 64);
@@ -193,12 +197,15 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
     total += x.size;
   }
 
+  // Tiles of at most 128 columns everywhere: the six-slot ring instance.
+  bool narrow = true;
+  for (const SplitProb& x : sp) narrow = narrow && x.bn <= kNarrowBN;
+
   // ---- bands, packing tasks, tiles ----
   std::vector<PackBand> bands;
   std::vector<int> band_prob, band_isa;  // host only: each band's problem and operand
   std::vector<int> task_band;
-  std::vector<int4> split_items;
-  std::vector<GroupDev> gdev(sp.size());
+  std::vector<TileJob> jobs;
   int64_t amax_words = 0, n_cnt = 0;
   for (size_t i = 0; i < sp.size(); ++i) {
     amax_words += probs[sp[i].g].m + probs[sp[i].g].n;
@@ -216,10 +223,6 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
   for (size_t i = 0; i < sp.size(); ++i) {
     const SplitProb& x = sp[i];
     const gbgemm_problem& q = probs[x.g];
-    GroupDev& d = gdev[i];
-    d.m = q.m; d.n = q.n; d.nkc = x.nkc; d.bn = x.bn; d.rowsA = x.rowsA; d.rowsB = x.rowsB;
-    d.parts = x.parts;
-    d.alpha = q.alpha; d.beta = q.beta; d.C = q.C; d.ldc = q.ldc;
     // bands in the order of the first tile that reads them (tiles go column
     // of tiles by column of tiles): op(B)'s bands of tile column 0, every
     // band of op(A), the remaining bands of op(B)
@@ -247,13 +250,28 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
     for (int j = 0; j < nb0; ++j) add_band(false, j);
     for (int j = 0; j < x.ra; ++j) add_band(true, j);
     for (int j = nb0; j < x.rb; ++j) add_band(false, j);
+    TileJob d{};  // the panels and maxima are filled in once the device memory is there
+    d.a_kstride = (size_t)x.rowsA * 128;
+    d.b_kstride = (size_t)x.rowsB * 128;
+    d.nkc = x.nkc; d.bn = x.bn; d.parts = x.parts;
+    d.m = q.m; d.n = q.n;
+    d.C = q.C; d.ldc = q.ldc; d.alpha = q.alpha; d.beta = q.beta;
     const int tn = (int)((q.n + x.bn - 1) / x.bn);
-    for (int c = 0; c < tn; ++c)
-      for (int r = 0; r < x.ra; ++r) split_items.push_back(make_int4((int)i, r, c, 0));
+    for (int c = 0; c < tn; ++c) {
+      d.n0 = (int64_t)c * x.bn;
+      d.b_rows = (int)std::min<int64_t>(x.bn, (q.n - d.n0 + 15) / 16 * 16);
+      for (int r = 0; r < x.ra; ++r) {
+        d.m0 = (int64_t)r * 128;
+        d.a_rows = (int)std::min<int64_t>(128, x.rowsA - d.m0);
+        // chunks that share a ring slot
+        d.group = std::max(1, std::min(128 / d.a_rows, (narrow ? kNarrowBN : kMaxBN) / d.b_rows));
+        jobs.push_back(d);
+      }
+    }
     cnt_base += x.ra + x.rb;
     aw += q.m + q.n;
   }
-  if (task_band.size() > 0x7FFFFFFF || split_items.size() > 0x7FFFFFFF) return GBGEMM_ERR_INVALID_VALUE;
+  if (task_band.size() > 0x7FFFFFFF || jobs.size() > 0x7FFFFFFF) return GBGEMM_ERR_INVALID_VALUE;
   std::vector<int4> simt_items[3 * 8];  // index: config * 8 + variant
   for (size_t s = 0; s < sprobs.size(); ++s) {
     int bm, bn;
@@ -268,8 +286,7 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
   }
   for (auto& v : simt_items)
     std::stable_sort(v.begin(), v.end(), [&](const int4& a, const int4& b) { return sprobs[a.x].k > sprobs[b.x].k; });
-  const Region gdev_r = take(gdev.size() * sizeof(GroupDev) + 16);
-  const Region sitems_r = take(split_items.size() * sizeof(int4) + 16);
+  const Region jobs_r = take(jobs.size() * sizeof(TileJob) + 16);
   const Region bands_r = take(bands.size() * sizeof(PackBand) + 16);
   const Region tband_r = take(task_band.size() * 4 + 16);
   const Region sprob_r = take(sprobs.size() * sizeof(Problem) + 16);
@@ -288,6 +305,8 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
   uint32_t* amax_base = reinterpret_cast<uint32_t*>(base + amax_r.off);
   aw = 0;
   std::vector<uint8_t*> pa(sp.size()), pb(sp.size()), pa2(sp.size()), pb2(sp.size());
+  std::vector<uint32_t*> amax(sp.size());  // op(A)'s maxima, then op(B)'s
+  size_t tj = 0;
   for (size_t i = 0; i < sp.size(); ++i) {
     const SplitProb& x = sp[i];
     const gbgemm_problem& q = probs[x.g];
@@ -296,28 +315,30 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
     pb[i] = r0 + x.offB;
     pa2[i] = x.parts == 2 ? r0 + x.offA2 : nullptr;
     pb2[i] = x.parts == 2 ? r0 + x.offB2 : nullptr;
-    GroupDev& d = gdev[i];
-    d.panelA = pa[i];
-    d.panelB = pb[i];
-    d.a_part = x.parts == 2 ? (int64_t)(pa2[i] - pa[i]) : 0;
-    d.b_part = x.parts == 2 ? (int64_t)(pb2[i] - pb[i]) : 0;
-    d.amaxA = amax_base + aw;
-    d.amaxB = amax_base + aw + q.m;
+    amax[i] = amax_base + aw;
     aw += q.m + q.n;
+    for (int t = 0; t < x.tiles; ++t, ++tj) {
+      TileJob& d = jobs[tj];
+      d.a_src = pa[i] + (size_t)d.m0 * 128;
+      d.b_src = pb[i] + (size_t)d.n0 * 128;
+      d.a_part = x.parts == 2 ? (int64_t)(pa2[i] - pa[i]) : 0;
+      d.b_part = x.parts == 2 ? (int64_t)(pb2[i] - pb[i]) : 0;
+      d.amaxA = amax[i];
+      d.amaxB = amax[i] + q.m;
+    }
   }
   for (size_t bi = 0; bi < bands.size(); ++bi) {
     PackBand& b = bands[bi];
     const int i = band_prob[bi];
     const bool is_a = band_isa[bi] != 0;
-    b.amax = const_cast<uint32_t*>(is_a ? gdev[i].amaxA : gdev[i].amaxB);
+    b.amax = amax[i] + (is_a ? 0 : probs[sp[i].g].m);
     b.panel = is_a ? pa[i] : pb[i];
     b.panel2 = is_a ? pa2[i] : pb2[i];
   }
   auto h2d = [&](const Region& r, const void* src, size_t bytes) {
     return bytes == 0 || cudaMemcpy(base + r.off, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
   };
-  bool ok = h2d(gdev_r, gdev.data(), gdev.size() * sizeof(GroupDev)) &&
-            h2d(sitems_r, split_items.data(), split_items.size() * sizeof(int4)) &&
+  bool ok = h2d(jobs_r, jobs.data(), jobs.size() * sizeof(TileJob)) &&
             h2d(bands_r, bands.data(), bands.size() * sizeof(PackBand)) &&
             h2d(tband_r, task_band.data(), task_band.size() * 4) &&
             h2d(sprob_r, sprobs.data(), sprobs.size() * sizeof(Problem));
@@ -325,14 +346,11 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
   if (!ok) return GBGEMM_ERR_CUDA;
   P->n_split = (int64_t)sp.size();
   P->n_simt = (int64_t)sprobs.size();
-  P->split_tiles = (int64_t)split_items.size();
+  P->split_tiles = (int64_t)jobs.size();
   P->kernels_per_run = 0;
 
   // ---- capture the graph ----
-  // Tiles of at most 128 columns everywhere: the six-slot ring instance.
-  bool narrow = true;
-  for (const GroupDev& gd : gdev) narrow = narrow && gd.bn <= kNarrowBN;
-  if (!gdev.empty()) {
+  if (!sp.empty()) {
     const cudaError_t ea = narrow ? ensure_gemm_smem_attr<GroupedSched, kNarrowStages, kNarrowBN>()
                                   : ensure_gemm_smem_attr<GroupedSched>();
     if (ea != cudaSuccess) return GBGEMM_ERR_CUDA;
@@ -383,21 +401,20 @@ int build_grouped_plan(GroupedPlan* P, const gbgemm_problem* probs, int64_t coun
     ++simt_launches;
   }
   P->kernels_per_run += simt_launches;
-  if (!gdev.empty() && e == cudaSuccess) {
+  if (!sp.empty() && e == cudaSuccess) {
     e = cudaMemsetAsync(base, 0, head_bytes, capture_stream);
     GroupedSched S;
     S.ctl = reinterpret_cast<WorkCtl*>(base + ctl_r.off);
     S.band_cnt = reinterpret_cast<int*>(base + cnt_r.off);
-    S.items = reinterpret_cast<const int4*>(base + sitems_r.off);
-    S.groups = reinterpret_cast<const GroupDev*>(base + gdev_r.off);
+    S.jobs = reinterpret_cast<const TileJob*>(base + jobs_r.off);
     S.bands = reinterpret_cast<const PackBand*>(base + bands_r.off);
     S.task_band = reinterpret_cast<const int*>(base + tband_r.off);
-    S.n_items = (int)split_items.size();
+    S.n_items = (int)jobs.size();
     S.n_tasks = (int)task_band.size();
     if (e == cudaSuccess) {
       // every packing task as its own CTA, then the GEMM
       pack_tasks_kernel<GroupedSched><<<(unsigned)task_band.size(), 256, 0, capture_stream>>>(S);
-      const int grid = (int)std::min<int64_t>((int64_t)split_items.size(), P->num_sms);
+      const int grid = (int)std::min<int64_t>((int64_t)jobs.size(), P->num_sms);
       e = cudaGetLastError();
       if (e == cudaSuccess)
         e = narrow ? launch_gemm_kernel<GroupedSched, kNarrowStages, kNarrowBN>(S, grid, P->status, capture_stream, true)

@@ -260,17 +260,23 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile i
 }
 
 // mbar_wait with suspending polls (see mbar_try_hint); same limits.
-__device__ __noinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                             uint64_t timeout_ns, uint32_t hint_ns) {
-  if (mbar_try(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
+  uint64_t t0 = 0;  // the clock starts at the eighth try: most waits end before it
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_hint(bar, parity, hint_ns)) return true;
     if ((it & 7u) == 0u) {
       if (*abort_flag) return false;
-      if (globaltimer() - t0 > timeout_ns) return false;
+      const uint64_t t = globaltimer();
+      if (t0 == 0) t0 = t;
+      if (t - t0 > timeout_ns) return false;
     }
   }
+}
+
+__device__ __forceinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               uint64_t timeout_ns, uint32_t hint_ns) {
+  return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, abort_flag, timeout_ns, hint_ns);
 }
 
 // Ask L2 for the 128-byte line holding `p`.
