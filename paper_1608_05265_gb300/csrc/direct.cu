@@ -40,6 +40,7 @@ double packed_us(int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bo
   if (s > 1) t += 5.0;
   const double chunks = std::ceil(nkc / s);
   if (bn == 256 && tm >= 2 && (!three || nkc >= 8)) {
+    if (s == 1) return t + choose_pair_tiles(m, n, batch, panel_k_chunks(k), three, num_sms / 2).us;
     const double items = (double)((tm + 1) / 2 * ((n + 255) / 256) * batch) * s;
     return t + std::ceil(items / (num_sms / 2)) * (chunks * (three ? 1.0 : 0.5) + 4.0);
   }

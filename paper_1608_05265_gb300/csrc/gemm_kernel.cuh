@@ -190,12 +190,13 @@ struct SingleSched {
   // of slice s, tile (tm, tn) at partial + ((s * tiles_m + tm) * tiles_n + tn) * 128 * bn
   int splitk, slice_chunks;
   float* partial;
-  // pair tiles (clusters of two CTAs, bn = 256): item t is a 256 x 256 tile
-  // (with split-K: one k slice of it), tile rows 2 tm2 and 2 tm2 + 1 of pair
-  // row tm2
-  int pair;
+  // pair tiles (clusters of two CTAs): item t is a 256 x bn tile (with
+  // split-K: one k slice of it), tile rows 2 tm2 and 2 tm2 + 1 of pair row
+  // tm2; from item tail_start on the tiles come in halves of bn / 2 columns
+  int pair, tail_start;
   __device__ __forceinline__ int num_items() const {
-    return (pair ? ((tiles_m + 1) >> 1) : tiles_m) * tiles_n * batch * splitk;
+    if (!pair) return tiles_m * tiles_n * batch * splitk;
+    return 2 * (((tiles_m + 1) >> 1) * tiles_n * batch * splitk) - tail_start;
   }
   __device__ __forceinline__ TileJob job(int t) const {
     const int per = tiles_m * tiles_n;
@@ -204,27 +205,37 @@ struct SingleSched {
     const int z = t / per;
     int tm, tn;
     tile_coords(t - z * per, tiles_m, tiles_n, raster, tm, tn);
-    return tile_job(z, tm, tn, sl, (int64_t)tn * bn);
+    return tile_job(z, tm, tn, sl, (int64_t)tn * bn, bn, bn, (int64_t)tn * bn);
   }
   // The half of pair item t that CTA `rank` of the pair computes: tile row
   // 2 tm2 + rank (the A panel has an even number of row blocks, so the odd
   // row of a last, half-empty pair reads the panel's padding block, which is
-  // never written; its rows lie past m and its epilogue stores nothing),
-  // B rows [n0 + 128 rank, n0 + 128 rank + 128) for its share of the B
-  // operand, and the item's k slice.  Pair rows go in groups of
+  // never written; its rows lie past m and its epilogue stores nothing), its
+  // half of the op(B) rows that the tile's columns fill (a multiple of 32 in
+  // all, so never past the panel, whose rows are a multiple of 256; a half
+  // tile past n reads row 0 and stores nothing), and the item's k slice.  Pair rows go in groups of
   // raster / 2, the same rows of C as the single-CTA groups of `raster` tile
   // rows.
   __device__ __forceinline__ TileJob job_pair(int t, int rank) const {
     const int tiles_m2 = (tiles_m + 1) >> 1;
     const int per = tiles_m2 * tiles_n;
+    int width = bn, half = 0;
+    if (t >= tail_start) {
+      half = (t - tail_start) & 1;
+      t = tail_start + ((t - tail_start) >> 1);
+      width = bn >> 1;
+    }
     const int sl = t % splitk;
     t /= splitk;
     const int z = t / per;
     int tm2, tn;
     tile_coords(t - z * per, tiles_m2, tiles_n, raster > 1 ? raster >> 1 : 1, tm2, tn);
-    return tile_job(z, 2 * tm2 + rank, tn, sl, (int64_t)tn * bn + 128 * rank);
+    const int64_t n0 = (int64_t)tn * bn + half * width;
+    const int rows = (int)max((int64_t)32, min((int64_t)width, (n - n0 + 31) / 32 * 32));
+    return tile_job(z, 2 * tm2 + rank, tn, sl, n0, width, rows, (n0 < n ? n0 : 0) + (rows >> 1) * rank);
   }
-  __device__ __forceinline__ TileJob tile_job(int z, int tm, int tn, int sl, int64_t b_row0) const {
+  __device__ __forceinline__ TileJob tile_job(int z, int tm, int tn, int sl, int64_t n0, int width, int b_rows,
+                                              int64_t b_row0) const {
     const int kc0 = sl * slice_chunks;
     TileJob j;
     j.a_kstride = (size_t)rbA * kBlockBytes;
@@ -232,11 +243,11 @@ struct SingleSched {
     j.a_src = panelA + (size_t)z * ps + (size_t)tm * kBlockBytes + (size_t)kc0 * j.a_kstride;
     j.b_src = panel_rows(panelB + (size_t)z * ps, b_row0) + (size_t)kc0 * j.b_kstride;
     j.nkc = (nkc - kc0 < slice_chunks) ? nkc - kc0 : slice_chunks;
-    j.bn = bn;
-    j.a_rows = 128; j.b_rows = bn; j.group = 1;
+    j.bn = width;
+    j.a_rows = 128; j.b_rows = b_rows; j.group = 1;
     j.partial = splitk > 1 ? partial + ((size_t)(sl * tiles_m + tm) * tiles_n + tn) * 128 * bn : nullptr;
     j.parts = parts; j.a_part = a_part; j.b_part = b_part;
-    j.m0 = (int64_t)tm * 128; j.n0 = (int64_t)tn * bn;
+    j.m0 = (int64_t)tm * 128; j.n0 = n0;
     j.m = m; j.n = n;
     j.amaxA = amaxA + (size_t)z * as; j.amaxB = amaxB + (size_t)z * as;
     j.C = C + (size_t)z * cs; j.ldc = ldc; j.alpha = alpha; j.beta = beta;
@@ -873,7 +884,7 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       // wait, like the first columns' below
       const int64_t i = J.m0 + q * 32 + lane;
       const bool row_ok = i < J.m;
-      const int cols = (J.bn / (kEpiWarps / 4)) > 32 ? J.bn / (kEpiWarps / 4) : 32;
+      const int cols = (J.bn / (kEpiWarps / 4) + 31) / 32 * 32;
       const int c_begin = part * cols, c_end = (c_begin + cols < J.bn) ? c_begin + cols : J.bn;
       auto col_bits = [&](int c0) -> uint32_t {
         const int64_t jl = J.n0 + c0 + lane;

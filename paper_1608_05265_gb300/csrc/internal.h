@@ -96,6 +96,16 @@ inline size_t panel_bytes(int64_t rows, int64_t k) {
   return (size_t)panel_row_blocks(rows) * (size_t)panel_k_chunks(k) * (size_t)kBlockBytes;
 }
 
+// The tiles of a pair launch (256 rows x bn columns, clusters of two CTAs on
+// `pairs` pairs of SMs): the width that fills the rounds of the pairs best, and
+// the tile from which on they come in two halves (tiles: none).
+struct PairTiles {
+  int bn = 256;
+  int64_t tiles = 0, tail_start = 0;
+  double us = 0.0;  // estimated time of the launch
+};
+PairTiles choose_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks, bool three, int pairs);
+
 // Workspace of one split-path call (or strided batch), in bytes from its
 // start: [control words | band counters | row maxima | per problem: panel A,
 // panel B (and with three parts the compact lo3 panels A2, B2) | split-K

@@ -27,6 +27,8 @@
 //    C, and the epilogue writes each column's 128 rows with one coalesced
 //    warp store per 32 rows (Section III-D assigns each core whole column
 //    blocks of the result for the same reason).
+#include <algorithm>
+
 #include "gemm_kernel.cuh"
 
 namespace gbg {
@@ -226,10 +228,43 @@ SingleSched make_single_sched(const SplitCall& c, const SplitLayout& L) {
   S.slice_chunks = (S.nkc + S.splitk - 1) / S.splitk;
   S.partial = c.splitk > 1 ? reinterpret_cast<float*>(ws + L.partial_off) : nullptr;
   S.pair = 0;
+  S.tail_start = 0;
   return S;
 }
 
 }  // namespace
+
+// Estimated time of a tile of `w` columns: the MMAs of its k chunks (0.5 us a
+// chunk of 256 columns, twice that with three parts), or below about 205
+// columns the copies that feed them (a chunk's op(A) block is as large for
+// every width), and the fill and the way out.
+static double pair_tile_us(int w, int64_t chunks, bool three) {
+  const double wide = std::max((double)w, (16384.0 + 64.0 * w) / 144.0) / 256.0;
+  return (double)chunks * (three ? 1.0 : 0.5) * wide + 1.0 + 3.0 * w / 256.0;
+}
+
+// With 256 columns throughout, the last round of tiles is often nearly empty
+// (4096^2: 256 tiles on 76 pairs, 3.37 rounds; 1931 x 1207: 40 tiles) while a
+// narrower tile, or halves of the last ones, fills it.  Measured against 256
+// throughout: 1931 x 1207 x 877 35.6 -> 34.0 us (160 columns, 64 tiles),
+// 4096^3 298.7 -> 293.4 us (224 columns, exactly four rounds), 8192^3 the same
+// within 0.1% (halves for the last 36 tiles; bound by power).
+PairTiles choose_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks, bool three, int pairs) {
+  PairTiles best;
+  const int64_t rows = (m + 255) / 256 * batch;
+  for (int w = 256; w >= 64; w -= 32) {
+    const int64_t tiles = rows * ((n + w - 1) / w), tail = tiles % pairs;
+    const double whole = (double)(tiles - tail) / pairs * pair_tile_us(w, chunks, three);
+    auto offer = [&](int64_t tail_start, double us) {
+      if (best.tiles != 0 && us >= 0.99 * best.us) return;
+      best.bn = w; best.tiles = tiles; best.tail_start = tail_start; best.us = us;
+    };
+    offer(tiles, whole + (tail ? pair_tile_us(w, chunks, three) : 0.0));
+    if (tail && w % 64 == 0)
+      offer(tiles - tail, whole + (double)((2 * tail + pairs - 1) / pairs) * pair_tile_us(w / 2, chunks, three));
+  }
+  return best;
+}
 
 cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
   if (c.m <= 0 || c.k <= 0 || c.batch <= 0) return cudaSuccess;
@@ -270,18 +305,28 @@ cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
   if (e != cudaSuccess || items == 0) return e;
   const int grid = (int)(items < sms ? items : sms);
   const bool timed = c.gemm_begin && c.gemm_end;
-  // Pair tiles (clusters of two CTAs, 256 x 256 tiles) for the widest tiles
+  // Pair tiles (clusters of two CTAs, tiles of 256 rows) for the widest tiles
   // of calls with at least two tile rows; with three-part panels (k < 512)
   // only from 8 k chunks: below that a tile's MMAs take less time than its
   // epilogue, and pairing two CTAs' epilogues (and the fixed tile order) cost
   // more than the halved operand loads gain (k = 128: 21% slower at 16384^2).
-  const int64_t pair_items = (tm + 1) / 2 * tn * c.batch * splitk;
   const bool pair_ok = !c.pack_only && c.bn == 256 && tm >= 2 && (S.parts == 1 || S.nkc >= 8);
   const int pair_cap = !pair_ok ? 0
                        : S.parts == 2 ? gemm_pair_capacity<SingleSched, true>() : gemm_pair_capacity<SingleSched>();
   if (timed && (e = cudaEventRecord(c.gemm_begin, s)) != cudaSuccess) return e;
   if (pair_cap > 0) {
     S.pair = 1;
+    int64_t pair_items = (tm + 1) / 2 * tn * c.batch * splitk;
+    S.tail_start = (int)pair_items;
+    if (splitk == 1) {
+      const PairTiles T = choose_pair_tiles(c.m, c.n, c.batch, nkc, S.parts == 2, pair_cap);
+      if (2 * T.tiles <= (int64_t)0x7FFFFFFF) {
+        S.bn = T.bn;
+        S.tiles_n = (int)((c.n + T.bn - 1) / T.bn);
+        S.tail_start = (int)T.tail_start;
+        pair_items = 2 * T.tiles - T.tail_start;
+      }
+    }
     const int pairs = (int)(pair_items < pair_cap ? pair_items : pair_cap);
     e = S.parts == 2 ? launch_gemm_kernel_pair<SingleSched, true>(S, pairs, c.status, s, ptasks > 0 && !timed)
                      : launch_gemm_kernel_pair<SingleSched>(S, pairs, c.status, s, ptasks > 0 && !timed);
