@@ -380,7 +380,7 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
   if (rc != GBGEMM_OK) return rc;
   c.bn = split_bn; c.raster = d.raster; c.splitk = splitk;
   c.ws = h->ws;
-  h->kernel_launches += 1;  // the packing launch (the memset of the workspace head is not a kernel of ours)
+  h->kernel_launches += 1;  // the packing launch (the clearing of the workspace head is not counted)
   if (prof_pair(h, &c.gemm_begin, &c.gemm_end) != cudaSuccess) return GBGEMM_ERR_CUDA;
   if (gbg::launch_split_call(c, h->stream) != cudaSuccess) return GBGEMM_ERR_CUDA;
   h->kernel_launches += splitk > 1 ? 2 : 1;

@@ -440,6 +440,9 @@ __device__ __forceinline__ void pack_task_regs(const PackJob& P, uint32_t* smax)
     if (mxr[it] != 0u) atomicMax(&smax[rr], mxr[it]);
   }
   __syncthreads();
+  // the maxima and band counters are zero from here on (launched ahead of the
+  // kernel that clears them; nothing to wait for otherwise)
+  wait_prerequisite_grid();
   if (tid < 128 && r0 + tid < P.rows && smax[tid] != 0u) atomicMax(&P.amax[r0 + tid], smax[tid]);
 }
 

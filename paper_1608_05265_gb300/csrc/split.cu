@@ -266,6 +266,20 @@ PairTiles choose_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks,
   return best;
 }
 
+namespace {
+
+// The head of the workspace (control words, band counters, row maxima) set to
+// zero.  A kernel and not a memset, so that the packing can be launched ahead
+// of its end: a packing task needs the zeros only once it has its maxima.
+// 1931 x 1207 x 877 33.9 -> 31.3 us, 8192^2 x 128 120.6 -> 118.3 us.
+__global__ void __launch_bounds__(256) clear_head_kernel(uint4* __restrict__ p, int64_t n16) {
+  launch_dependents();
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n16; i += (int64_t)gridDim.x * 256)
+    p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+}  // namespace
+
 cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
   if (c.m <= 0 || c.k <= 0 || c.batch <= 0) return cudaSuccess;
   if (c.n < 0 || (c.n == 0 && !c.pack_only)) return cudaSuccess;
@@ -291,7 +305,16 @@ cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
   }
   // no empty slice (an empty slice would store a stale accumulator)
   if ((int64_t)(S.splitk - 1) * S.slice_chunks >= S.nkc) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(c.ws, 0, L.head, s);
+  const int64_t head16 = (int64_t)(L.head / 16);
+  const bool ahead = !c.pack_only && ptasks > 0 && L.head % 16 == 0;
+  cudaError_t e = cudaSuccess;
+  if (ahead) {
+    clear_head_kernel<<<(unsigned)std::min<int64_t>((head16 + 255) / 256, 64), 256, 0, s>>>(
+        static_cast<uint4*>(c.ws), head16);
+    e = cudaGetLastError();
+  } else {
+    e = cudaMemsetAsync(c.ws, 0, L.head, s);
+  }
   if (e != cudaSuccess) return e;
   if (c.pack_only && c.amax_out) {
     e = cudaMemsetAsync(c.amax_out, 0, (size_t)c.m * 4, s);
@@ -300,8 +323,18 @@ cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
   const int64_t items = tm * tn * c.batch * splitk;
   const int64_t sms = c.num_sms > 0 ? c.num_sms : 148;
   // packing tasks first, each its own CTA, then the GEMM
-  if (ptasks > 0) pack_tasks_kernel<SingleSched><<<(unsigned)ptasks, 256, 0, s>>>(S);
-  e = cudaGetLastError();
+  if (ptasks > 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ptasks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ahead ? 1 : 0;
+    e = cudaLaunchKernelEx(&cfg, pack_tasks_kernel<SingleSched>, S);
+  }
   if (e != cudaSuccess || items == 0) return e;
   const int grid = (int)(items < sms ? items : sms);
   const bool timed = c.gemm_begin && c.gemm_end;
