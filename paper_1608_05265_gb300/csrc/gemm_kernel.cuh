@@ -13,11 +13,11 @@
 // band's counter, and the task that completes a band re-packs the band's
 // badly scaled rows.  The GEMM launch follows on the same stream.
 //
-// GEMM roles (one CTA per SM, 608 threads):
+// GEMM roles (one CTA per SM, 608 threads, 640 with staged jobs):
 //   warp 0, lane 0  producer: takes the next tile from a device-wide counter
 //                   (dynamic scheduling, so the CTAs that run finish the
 //                   work however many are resident), hands its index to the
-//                   other roles through a four-slot queue in shared memory,
+//                   other roles through a queue in shared memory,
 //                   and streams one bulk async copy of the 128-row A block
 //                   and one of the BN B rows per 32-deep k chunk into the
 //                   stage ring ("full" mbarriers);
@@ -37,26 +37,30 @@
 //                   blocks of the result so that stores stay contiguous);
 //   warp 18         with beta != 0 and k <= 512, asks L2 for each tile's C
 //                   columns as soon as the tile is handed out, so that the
-//                   epilogue's reads of C find them there.  With staged jobs
-//                   (many problems) it also draws the tiles and leaves each
-//                   tile's job in shared memory, ahead of the producer.
+//                   epilogue's reads of C find them there;
+//   warp 19         with staged jobs (many problems) draws the tiles and
+//                   leaves each tile's job in shared memory, ahead of the
+//                   producer (else idle).
 //
 // What bounds the many-problem instance is the two single-thread roles: at
 // 4096 problems up to 1024^3 the issuer spent about 80 cycles per MMA and the
 // producer about 330 per bulk copy against 32-128 cycles of tensor time per
-// MMA, and 1 KB copies or no stores at all changed the time by 3%.  Hence
+// MMA, and 1 KB copies or no stores at all changed the time by 1 and 6%.  Hence
 // tiles of up to 256 columns (half the MMAs and copies per result), edge
 // tiles that copy and multiply only the rows that exist, several chunks of a
-// small tile per ring slot, descriptors advanced by additions, and waits
-// whose first poll is inline: 1975 us for the packing and the GEMM became
-// 1709 us (4096^3: 317 -> 301 us, 8192^3: 2102 -> 2019 us by the last two
-// and by the epilogue's maxima being read before its wait).  Asking L2 for
-// the panels ahead of the copies did not help (2015 us).
+// small tile per ring slot, descriptors advanced by additions, waits whose
+// first poll is inline, and a warp of its own that draws the tiles: packing and
+// GEMM 1989 -> 1671 us (GEMM 1075 -> 784), 128 problems up to 256 28.8 -> 28.3,
+// 2200 up to 512 with C read 489 -> 432.  (4096^3 317 -> 301 us and 8192^3
+// 2102 -> 2019 us by the cheaper issue and by the epilogue's maxima being read
+// before its wait.)  Asking L2 for the panels ahead of the copies did not help.
 // Every wait is bounded: on expiry the kernel records GBGEMM_ERR_DEVICE_TIMEOUT,
 // raises a CTA-wide abort flag, drains its own copies and MMAs, frees TMEM
 // and returns.  Waiting threads sleep (mbarrier try_wait with a suspend
 // hint) instead of spinning.
 #pragma once
+
+#include <type_traits>
 
 #include "split_device.cuh"
 
@@ -70,8 +74,11 @@ constexpr int kNarrowBN = 128;
 constexpr int kPairStages = 6;                     // ring depth of the pair-tile instance (half the B rows per CTA)
 constexpr int kEpiWarps = 16;
 constexpr int kCpfWarp = 2 + kEpiWarps;            // the C prefetch warp
-constexpr int kGemmThreads = 32 * (kCpfWarp + 1);  // 19 warps, charged as 20: 96 registers per thread
-constexpr int kTileQ = 4;                          // tile-index queue between the roles
+// 19 warps, charged as 20: 96 registers per thread.  With staged jobs the
+// twentieth draws the tiles.
+constexpr int gemm_threads(bool staged) { return 32 * (kCpfWarp + 1 + (staged ? 1 : 0)); }
+constexpr int kTileQ = 8;                          // tile queue between the roles
+constexpr int kAheadTiles = 3;                     // tiles handed out ahead of the producer at most
 constexpr int kAheadChunks = 6;                    // k chunks of tiles handed out ahead of the producer
 constexpr int kPackChunks = 4;                     // k chunks per packing task
 constexpr uint64_t kTimeoutNs = 2000000000ull;
@@ -487,7 +494,7 @@ __global__ void __launch_bounds__(256, 4) pack_tasks_kernel(const Sched S) {
 // fixed order (cluster c: items c, c + clusters, ...), so both CTAs of a
 // pair walk the same tiles without exchanging indices.
 template <class Sched, int STAGES = kStages, int MAXBN = kMaxBN, bool PAIR = false, bool THREE = false>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(Sched::kStagedJobs && !PAIR), 1)
 split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
   constexpr uint32_t A_BYTES = kBlockBytes;        // 128 rows x 128 B
   constexpr uint32_t B_STAGE = (PAIR ? MAXBN / 2 : MAXBN) * 128;  // room for the B rows of a stage
@@ -529,10 +536,12 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
   // Staged jobs: the scheduler warp leaves each tile's job in shared memory.
   constexpr bool STAGED = Sched::kStagedJobs && !PAIR;
   __shared__ TileJob job_q[STAGED ? kTileQ : 1];
-  auto take_job = [&](int slot, int t) -> TileJob {
+  auto take_job = [&](int slot, int t) -> std::conditional_t<STAGED, const TileJob&, TileJob> {
     if constexpr (STAGED) return job_q[slot];
     else return job_of(t);
   };
+  // Among the last tiles none is drawn before the tile before it has been read.
+  const int calm = num_items - 3 * (int)gridDim.x;
   auto wait_bar = [&](uint32_t bar, uint32_t parity) -> bool {
     return mbar_wait_hint(bar, parity, abort_flag, timeout_ns, kHintNs);
   };
@@ -542,11 +551,11 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), full_count); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), (PAIR ? 2 : 1) * kEpiWarps); }
     mbar_init(drain_bar, 1);
-    // a tile slot is read by the epilogue warps, the MMA issuer and one more:
-    // the producer where the scheduler warp fills it, else the prefetch warp
+    // a tile slot is read by the epilogue warps, the MMA issuer and the prefetch
+    // warp, and by the producer where it does not fill it itself
     for (int s = 0; s < kTileQ; ++s) {
       mbar_init(tqf_bar(s), 1);
-      mbar_init(tqe_bar(s), 2 + kEpiWarps);
+      mbar_init(tqe_bar(s), 2 + kEpiWarps + (STAGED ? 1 : 0));
       mbar_init(tqs_bar(s), 1);
     }
     *abort_flag = 0;
@@ -625,8 +634,9 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
         }
         if (t < 0) break;
         const TileJob J = take_job(tq, t);
+        const uint32_t begun_bar = tqs_bar(tq);
         if constexpr (STAGED) {
-          mbar_arrive(tqs_bar(tq));
+          if (t < calm) mbar_arrive(begun_bar);
           mbar_arrive(tqe_bar(tq));
         }
         if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
@@ -668,6 +678,9 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
             }
             if (++stage == kStages) { stage = 0; phase ^= 1u; wrapped = true; }
           }
+        }
+        if constexpr (STAGED) {
+          if (t >= calm) mbar_arrive(begun_bar);
         }
       }
       // Let every copy this thread started land before the CTA can exit: the
@@ -757,7 +770,8 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
           break;
         }
         const int t = tile_q[tq];
-        const TileJob J = t < 0 ? TileJob{} : take_job(tq, t);
+        TileJob J;
+        if (t >= 0) J = take_job(tq, t);
         mbar_arrive(tqe_bar(tq));
         if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
         if (t < 0) break;
@@ -877,11 +891,10 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       }
       if (t < 0) break;
       if constexpr (STAGED) __syncwarp();  // lane 0 has seen the job complete
-      const TileJob J = take_job(tq, t);
-      if constexpr (STAGED) {
-        __syncwarp();  // every lane has read it
-        if (lane == 0) mbar_arrive(tqe_bar(tq));
-      }
+      // A staged job stays in shared memory, read where it is used (its fields
+      // in registers made the epilogue spill), and is given back at the end.
+      std::conditional_t<STAGED, const TileJob&, const TileJob> J = take_job(tq, t);
+      const uint32_t done_bar = tqe_bar(tq);
       if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
       // maxima were built by the packing: read them through L2, before the
       // wait, like the first columns' below
@@ -967,6 +980,7 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       }
       tc_fence_before();
       __syncwarp();
+      if (STAGED && lane == 0) mbar_arrive(done_bar);
       if (lane == 0) {
         // the accumulator buffer is free again: rank 0's MMA issuer waits for
         // both CTAs' epilogue warps of a pair
@@ -976,23 +990,62 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
       if (++abuf == 2) { abuf = 0; aphase ^= 1u; }
     }
   } else if (warp == kCpfWarp) {
-    // ---------------- C prefetch; staged jobs: also the tile scheduler ----------------
+    // ---------------- C prefetch ----------------
     // With beta != 0 the epilogue reads the tile's C: ask L2 for it as soon
     // as the tile is handed out, one to three tiles ahead of the epilogue.
-    // With staged jobs this warp draws the tiles: the counter and the job are
-    // two dependent trips to L2 or memory, which the producer and the MMA
-    // issuer each waited for at every tile.  It stays ahead of the producer
-    // by one tile, or by up to three while those hold fewer than kAheadChunks
-    // k chunks together, so that a CTA never sits on work others could do.
     int tq = 0;
     uint32_t tqph = 0;
-    int sq = 0, ahead = 0, ahead_chunks = 0;  // lane 0, staged: tiles the producer has not begun
-    uint32_t sqph = 0;
     for (;;) {
       int ok = 1, t = -1;
+      if (lane == 0) {
+        ok = mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs) ? 1 : 0;
+        if (ok) {
+          t = tile_q[tq];
+          if (!STAGED || t < 0) mbar_arrive(tqe_bar(tq));
+        }
+      }
+      ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+      t = __shfl_sync(0xFFFFFFFFu, t, 0);
+      if (!ok || t < 0) break;
+      if constexpr (STAGED) __syncwarp();  // lane 0 has seen the job complete
+      const TileJob J = take_job(tq, t);
       if constexpr (STAGED) {
+        __syncwarp();  // every lane has read it
+        if (lane == 0) mbar_arrive(tqe_bar(tq));
+      }
+      if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
+      // Only short tiles (k <= 512), whose epilogue rather than their MMAs
+      // sets the pace, are prefetched: for long ones the C reads overlap the
+      // next tile's MMAs anyway, and prefetching several 128 KB tiles ahead
+      // would push the operand panels out of L2.
+      if (J.beta == 0.f || J.partial || J.nkc > 16 || J.m0 >= J.m) continue;
+      const int64_t rows = (J.m - J.m0 < 128) ? J.m - J.m0 : 128;
+      const int64_t ncols = (J.n - J.n0 < J.bn) ? J.n - J.n0 : J.bn;
+      const float* c0 = J.C + J.m0 + J.n0 * J.ldc;
+      for (int64_t j = lane; j < ncols; j += 32) {
+        const char* col = reinterpret_cast<const char*>(c0 + j * J.ldc);
+        for (int64_t off = 0; off < rows * 4; off += 128) prefetch_l2(col + off);
+        prefetch_l2(col + rows * 4 - 4);
+      }
+    }
+  } else if (STAGED) {
+    // ---------------- tile scheduler (staged jobs) ----------------
+    // Draws the tiles and leaves their jobs in shared memory: the counter and
+    // the job are two dependent trips to L2 or memory, which the producer and
+    // the MMA issuer each waited for at every tile.  It stays ahead of the
+    // producer by one tile, or by up to three while those hold fewer than
+    // kAheadChunks k chunks together; at the end (from `calm` on) it draws a
+    // tile only when the one before has been read, so that no CTA sits on work
+    // that others could do.
+    if constexpr (STAGED) {
+      int tq = 0, last = -1;
+      uint32_t tqph = 0;
+      int sq = 0, ahead = 0, ahead_chunks = 0;  // lane 0: tiles the producer has not begun (at the end: not read)
+      uint32_t sqph = 0;
+      for (;;) {
+        int ok = 1, t = -1;
         if (lane == 0) {
-          while (ok && ahead > 0 && (ahead_chunks >= kAheadChunks || ahead == kTileQ - 1)) {
+          while (ok && ahead > 0 && (last >= calm || ahead_chunks >= kAheadChunks || ahead == kAheadTiles)) {
             ok = wait_bar(tqs_bar(sq), sqph) ? 1 : 0;
             --ahead;
             ahead_chunks -= job_q[sq].nkc;
@@ -1020,34 +1073,10 @@ split_gemm_kernel(const Sched S, int* status, uint64_t timeout_ns) {
           mbar_arrive(tqf_bar(tq));
         }
         if (t < 0) break;
+        last = t;
         ++ahead;
         ahead_chunks += job_q[tq].nkc;
-      } else {
-        if (lane == 0) {
-          ok = mbar_wait_hint(tqf_bar(tq), tqph, abort_flag, timeout_ns, kHintNs) ? 1 : 0;
-          if (ok) {
-            t = tile_q[tq];
-            mbar_arrive(tqe_bar(tq));
-          }
-        }
-        ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-        t = __shfl_sync(0xFFFFFFFFu, t, 0);
-        if (!ok || t < 0) break;
-      }
-      const TileJob J = take_job(tq, t);
-      if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
-      // Only short tiles (k <= 512), whose epilogue rather than their MMAs
-      // sets the pace, are prefetched: for long ones the C reads overlap the
-      // next tile's MMAs anyway, and prefetching several 128 KB tiles ahead
-      // would push the operand panels out of L2.
-      if (J.beta == 0.f || J.partial || J.nkc > 16 || J.m0 >= J.m) continue;
-      const int64_t rows = (J.m - J.m0 < 128) ? J.m - J.m0 : 128;
-      const int64_t ncols = (J.n - J.n0 < J.bn) ? J.n - J.n0 : J.bn;
-      const float* c0 = J.C + J.m0 + J.n0 * J.ldc;
-      for (int64_t j = lane; j < ncols; j += 32) {
-        const char* col = reinterpret_cast<const char*>(c0 + j * J.ldc);
-        for (int64_t off = 0; off < rows * 4; off += 128) prefetch_l2(col + off);
-        prefetch_l2(col + rows * 4 - 4);
+        if (++tq == kTileQ) { tq = 0; tqph ^= 1u; }
       }
     }
   }
@@ -1093,7 +1122,7 @@ cudaError_t launch_gemm_kernel(const Sched& S, int grid, int* status, cudaStream
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(gemm_threads(Sched::kStagedJobs));
   cfg.dynamicSmemBytes = gemm_smem_bytes<STAGES, MAXBN>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -1119,7 +1148,7 @@ int gemm_pair_capacity() {
     if (ensure_gemm_smem_attr<Sched, kPairStages, kMaxBN, true, THREE>() == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2);
-      cfg.blockDim = dim3(kGemmThreads);
+      cfg.blockDim = dim3(gemm_threads(false));
       cfg.dynamicSmemBytes = gemm_smem_bytes<kPairStages, kMaxBN, true>();
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1146,7 +1175,7 @@ cudaError_t launch_gemm_kernel_pair(const Sched& S, int pairs, int* status, cuda
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * pairs));
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(gemm_threads(false));
   cfg.dynamicSmemBytes = gemm_smem_bytes<kPairStages, kMaxBN, true>();
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
