@@ -45,8 +45,9 @@
 // its exponent is taken from the first step in which it is not all zero
 // (until then everything it contributed is zero, so the exponent may still
 // be set), and the rest of the vector is watched: an element that comes out
-// at 2^50 or more after scaling makes the CTA (the pair's cluster) compute
-// its slice again with exponents from the true maxima.  Within those limits
+// at 2^50 or more after scaling, or beyond FP32, makes the CTA (the pair's
+// cluster) compute its slice again with exponents from the true maxima.
+// Within those limits
 // the result is what exponents from the true maxima give: powers of two
 // commute with FP32 rounding, and products stay within 2^100.  Every slice
 // scales on its own; the sum of the slices brings their accumulators to the
@@ -213,12 +214,19 @@ struct Operand {
       }
     }
   }
-  __device__ __forceinline__ void scale(float (&v)[N], const int* ex) const {
+  // Whether a finite value left FP32's range (its vector's exponent, taken
+  // from an earlier step, is far too small for it).
+  __device__ __forceinline__ bool scale(float (&v)[N], const int* ex) const {
+    bool left = false;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       const int e = ex[row_of(j)];
-      if (e != 0 && isfinite(v[j])) v[j] = scale_pow2(v[j], e);
+      if (e != 0 && isfinite(v[j])) {
+        v[j] = scale_pow2(v[j], e);
+        left |= !isfinite(v[j]);
+      }
     }
+    return left;
   }
   // Split the chunk and store it; returns the largest finite |v|.  One test
   // for Inf and NaN per chunk keeps the usual case one run of independent
@@ -527,8 +535,8 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
         open = __syncthreads_or(mine) != 0;
       }
       if (scaled) {
-        OA.scale(a, exA);
-        OB.scale(b, exBo);
+        const bool left_a = OA.scale(a, exA), left_b = OB.scale(b, exBo);
+        if (left_a || left_b) top = INFINITY;
       }
       wait(empty_bar(stage), phase ^ 1u);
       uint8_t* const st = ring + stage * D::STAGE + sub * D::CHUNK;
