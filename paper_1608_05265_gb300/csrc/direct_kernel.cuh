@@ -42,17 +42,20 @@
 //
 // Scaling of badly scaled K-vectors (largest magnitude outside [2^-48,
 // 2^48)): a vector's maximum is not known before its elements are loaded, so
-// its exponent is taken from the first step in which it is not all zero
-// (until then everything it contributed is zero, so the exponent may still
-// be set), and the rest of the vector is watched: an element that comes out
-// at 2^50 or more after scaling, or beyond FP32, makes the CTA (the pair's
-// cluster) compute its slice again with exponents from the true maxima.
-// Within those limits
-// the result is what exponents from the true maxima give: powers of two
-// commute with FP32 rounding, and products stay within 2^100.  Every slice
-// scales on its own; the sum of the slices brings their accumulators to the
-// largest exponent of each row and column first, so that nothing is rounded
-// to a subnormal before the end.
+// its exponent is taken from the first step (none if it is zero there), and
+// the rest of the vector is watched: an element that comes out at 2^50 or
+// more after scaling, or beyond FP32, or a vector that was zero in the first
+// step and whose maximum then lies below 2^-48, makes the CTA (the pair's
+// cluster) compute its slice again with exponents from the true maxima.  The
+// last watch costs only the threads that hold such vectors, and no barrier
+// (512 x 512 x 65536 with every second row of op(A) zero, 129 -> 109 us
+// against 98 of dense operands; both operands k contiguous at ld + 1, 267 ->
+// 152 against 135; before, every step waited for the block's maxima while a
+// vector was zero).  Within those limits the result is what exponents from
+// the true maxima give: powers of two commute with FP32 rounding, and
+// products stay within 2^100.  Every slice scales on its own; the sum of the
+// slices brings their accumulators to the largest exponent of each row and
+// column first, so that nothing is rounded to a subnormal before the end.
 #pragma once
 
 #include "direct.h"
@@ -86,7 +89,8 @@ struct DirectShape {
   static constexpr int CTAS = PARTS == 3 ? 2 : 1;
   static constexpr int STAGES = 2;
   static constexpr int RING = STAGES * STAGE;
-  static constexpr int SMEM = RING + 1024 + 256 + 1536 + 1024;  // alignment, barriers, exponents, maxima
+  // alignment, barriers, exponents, maxima, every thread's late K-vectors
+  static constexpr int SMEM = RING + 1024 + 256 + 1536 + 1024 + 4 * THREADS;
   static constexpr int DEPTH = 2;  // steps in flight in registers
   static constexpr int TMEM = 2 * BN;  // accumulators: hi*hi, and the smaller products
   static_assert(CTAS * TMEM <= 512 && CTAS * (SMEM + 1024) <= 228 * 1024, "resident CTAs");
@@ -213,6 +217,52 @@ struct Operand {
         if ((threadIdx.x & 31) == 0) atomicMax(&rowmax[row_of(j)], b);
       }
     }
+  }
+  // The thread's rows: one (kRows), one of four values each (kVec), or one a
+  // value (kScalar, the same rows in every lane).  Bits of those that rowmax
+  // holds a zero for.
+  static constexpr int R = MODE == kRows ? 1 : MODE == kVec ? N / 4 : N;
+  static __device__ __forceinline__ uint16_t zero_rows(const uint32_t* rowmax) {
+    uint32_t bits = 0u;
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (rowmax[row_of(u * (N / R))] == 0u) bits |= 1u << u;
+    return (uint16_t)bits;
+  }
+  // The chunk's part in the maxima of the rows in *late, which loses the rows
+  // that turn out well scaled here.  Nobody waits for it: the maxima are read
+  // after the last step.
+  __device__ __forceinline__ void watch_rows(const float (&v)[N], uint16_t* late, uint32_t* rowmax) const {
+    const uint32_t bits = *late;
+    if (bits == 0u) return;
+    uint32_t seen = 0u;
+    if (MODE == kScalar) {  // a row's maximum is the warp's; mostly there is nothing but zeros
+      uint32_t any = 0u;
+#pragma unroll
+      for (int u = 0; u < N; ++u) any |= (bits >> u) & 1u ? __float_as_uint(v[u]) : 0u;
+      if (!__any_sync(0xFFFFFFFFu, (any & 0x7FFFFFFFu) != 0u)) return;
+      const int lane = threadIdx.x & 31;
+#pragma unroll
+      for (int u = 0; u < N; ++u)
+        if ((bits >> u) & 1u) {
+          const uint32_t b = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(v[u]) & 0x7FFFFFFFu);
+          if (b != 0u && lane == 0) atomicMax(&rowmax[row_of(u)], b);
+        }
+      __syncwarp();
+      seen = __ballot_sync(0xFFFFFFFFu, lane < N && rowmax[row_of(0) + min(lane, N - 1)] >= kWellScaledLo);
+    } else {
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        if (!((bits >> u) & 1u)) continue;
+        uint32_t b = 0u;
+#pragma unroll
+        for (int j = u * (N / R); j < (u + 1) * (N / R); ++j) b = max(b, __float_as_uint(v[j]) & 0x7FFFFFFFu);
+        if (b == 0u) continue;
+        atomicMax(&rowmax[row_of(u * (N / R))], b);
+        if (b >= kWellScaledLo) seen |= 1u << u;
+      }
+    }
+    if (bits & seen) *late = (uint16_t)(bits & ~seen);
   }
   // Whether a finite value left FP32's range (its vector's exponent, taken
   // from an earlier step, is far too small for it).
@@ -350,6 +400,11 @@ template <int BN, bool PAIR, int PARTS, int MA, int MB>
 __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectShape<BN, PAIR, PARTS>::CTAS) direct_gemm_kernel(const DirectArgs S) {
   using D = DirectShape<BN, PAIR, PARTS>;
   constexpr int BS = D::BS, UK = D::UK;
+  // With two parts, steps with K-vectors to watch have a loop of their own: its
+  // code in the one loop cost dense operands 1-6% of a call.  Not with two
+  // kScalar operands (two loops spill), nor with three parts (few steps).
+  constexpr bool OWN = PARTS == 2 && (MA != kScalar || MB != kScalar);
+  static_assert(D::DEPTH == 2, "steps alternate between two sets of registers");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
   uint8_t* const ring = smem_raw + (base - raw);
@@ -364,6 +419,7 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
   int* const exA = reinterpret_cast<int*>(tail + 256);          // exponents of the tile's 128 rows ...
   int* const exB = exA + 128;                                   // ... and BN columns
   uint32_t* const rowmax = reinterpret_cast<uint32_t*>(exB + 256);  // maxima: 128 rows, the BS columns split here
+  uint16_t* const late = reinterpret_cast<uint16_t*>(rowmax + 256 + threadIdx.x);  // this thread's: rows, columns
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   const bool clustered = PAIR || S.cluster_slices > 1;
@@ -494,9 +550,9 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
   for (;;) {
     const bool again = passes > 0;
     bool scaled = false;         // some K-vector split here has an exponent
-    bool open = true;            // some K-vector split here was zero so far
-    bool mine = tid < 128 + BS;  // this thread's K-vector (row tid, or column tid - 128) was
-    if (again) {                 // exponents from the true maxima of this slice
+    bool open = false;           // some K-vector split here was zero in the first step
+    bool mine = false;           // this thread's K-vector (row tid, or column tid - 128) was, at the end: throughout
+    if (again) {  // exponents from the true maxima of this slice
       __syncthreads();
       if (tid < 128 + BS) rowmax[tid] = 0u;
       __syncthreads();
@@ -513,26 +569,13 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
       if (tid < 128) exA[tid] = e;
       else if (tid < 128 + BS) exBo[tid - 128] = e;
       scaled = __syncthreads_or(e != 0);
-      open = false;
       load_first();
     }
     float top = 0.f;
-    auto step = [&](float (&a)[16], float (&b)[BS / 8], int i) {
-      if (open) {
-        // Exponents of the K-vectors whose first nonzero step this is.
-        OA.row_max(a, rowmax);
-        OB.row_max(b, rowmax + 128);
-        __syncthreads();
-        int e = 0;
-        if (mine && rowmax[tid] != 0u) {
-          e = scale_exp_from_bits(rowmax[tid]);
-          if (tid < 128) exA[tid] = e;
-          else exBo[tid - 128] = e;
-          mine = false;
-        }
-        if (tid < 128 + BS) rowmax[tid] = 0u;
-        scaled |= __syncthreads_or(e != 0) != 0;
-        open = __syncthreads_or(mine) != 0;
+    auto step = [&](float (&a)[16], float (&b)[BS / 8], int i, bool watch) {
+      if (watch) {
+        OA.watch_rows(a, late, rowmax);
+        OB.watch_rows(b, late + 1, rowmax + 128);
       }
       if (scaled) {
         const bool left_a = OA.scale(a, exA), left_b = OB.scale(b, exBo);
@@ -557,17 +600,49 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
       __syncwarp();
       if (++stage == D::STAGES) { stage = 0; phase ^= 1u; }
     };
-    for (int i = 0; i < steps; i += D::DEPTH) {
-#pragma unroll
-      for (int d = 0; d < D::DEPTH; ++d)
-        if (i + d < steps) step(va[d], vb[d], i + d);
+    if (!again) {  // exponents of the K-vectors that are not zero in the first step
+      OA.row_max(va[0], rowmax);
+      OB.row_max(vb[0], rowmax + 128);
+      __syncthreads();
+      int e = 0;
+      if (tid < 128 + BS) {
+        e = scale_exp_from_bits(rowmax[tid]);
+        if (tid < 128) exA[tid] = e;
+        else exBo[tid - 128] = e;
+        mine = rowmax[tid] == 0u;
+      }
+      scaled = __syncthreads_or(e != 0) != 0;
+      open = __syncthreads_or(mine) != 0;
+      if (open) {
+        late[0] = OA.zero_rows(rowmax);
+        late[1] = OB.zero_rows(rowmax + 128);
+        __syncthreads();  // every thread has its bits before the watch writes
+      }
     }
+    auto pass = [&](bool watch) {
+      for (int i = 0; i < steps; i += D::DEPTH) {
+#pragma unroll
+        for (int d = 0; d < D::DEPTH; ++d)
+          if (i + d < steps) step(va[d], vb[d], i + d, watch);
+      }
+    };
+    if (!OWN) pass(open);
+    else if (open) pass(true);
+    else pass(false);
     if (issuer) {
       if constexpr (PAIR) mma_commit_pair(accf, (uint16_t)(3u << lead));
       else mma_commit(accf);
     }
     __syncwarp();
-    const bool over = __syncthreads_or(!again && top >= kWatchLimit) != 0;
+    bool low = false;  // a K-vector that was zero in the first step is badly scaled after it
+    if (open) {
+      __syncthreads();  // the watched maxima are complete
+      if (mine) {
+        low = rowmax[tid] != 0u && rowmax[tid] < kWellScaledLo;
+        mine = rowmax[tid] == 0u;
+      }
+    }
+    const bool over = __syncthreads_or(!again && (top >= kWatchLimit || low)) != 0;
     if (tid == 0 && over) *redo_s = 1;
     if (tid == 0 && scaled) *scaled_s = 1;
     if (mine) (tid < 128 ? exA[tid] : exBo[tid - 128]) = kNoExp;
