@@ -46,7 +46,10 @@
 // the rest of the vector is watched: an element that comes out at 2^50 or
 // more after scaling, or beyond FP32, or a vector that was zero in the first
 // step and whose maximum then lies below 2^-48, makes the CTA (the pair's
-// cluster) compute its slice again with exponents from the true maxima.  The
+// cluster) compute its slice again with exponents from the true maxima.  Three
+// parts (at most 16 steps) take the exponent from the first step in which the
+// vector is not zero, with barriers until then: 4% on a call with zero vectors,
+// where the watch's code cost dense ones up to 5%.  With two parts the
 // last watch costs only the threads that hold such vectors, and no barrier
 // (512 x 512 x 65536 with every second row of op(A) zero, 129 -> 109 us
 // against 98 of dense operands; both operands k contiguous at ld + 1, 267 ->
@@ -550,8 +553,9 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
   for (;;) {
     const bool again = passes > 0;
     bool scaled = false;         // some K-vector split here has an exponent
-    bool open = false;           // some K-vector split here was zero in the first step
-    bool mine = false;           // this thread's K-vector (row tid, or column tid - 128) was, at the end: throughout
+    // some K-vector split here was zero in the first step (three parts: so far), and
+    // this thread's (row tid, or column tid - 128); at the end: throughout
+    bool open = PARTS == 3 && !again, mine = open && tid < 128 + BS;
     if (again) {  // exponents from the true maxima of this slice
       __syncthreads();
       if (tid < 128 + BS) rowmax[tid] = 0u;
@@ -573,9 +577,24 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
     }
     float top = 0.f;
     auto step = [&](float (&a)[16], float (&b)[BS / 8], int i, bool watch) {
-      if (watch) {
+      if (PARTS == 2 && watch) {
         OA.watch_rows(a, late, rowmax);
         OB.watch_rows(b, late + 1, rowmax + 128);
+      }
+      if (PARTS == 3 && open) {  // exponents of the K-vectors whose first nonzero step this is
+        OA.row_max(a, rowmax);
+        OB.row_max(b, rowmax + 128);
+        __syncthreads();
+        int e = 0;
+        if (mine && rowmax[tid] != 0u) {
+          e = scale_exp_from_bits(rowmax[tid]);
+          if (tid < 128) exA[tid] = e;
+          else exBo[tid - 128] = e;
+          mine = false;
+        }
+        if (tid < 128 + BS) rowmax[tid] = 0u;
+        scaled |= __syncthreads_or(e != 0) != 0;
+        open = __syncthreads_or(mine) != 0;
       }
       if (scaled) {
         const bool left_a = OA.scale(a, exA), left_b = OB.scale(b, exBo);
@@ -600,7 +619,7 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
       __syncwarp();
       if (++stage == D::STAGES) { stage = 0; phase ^= 1u; }
     };
-    if (!again) {  // exponents of the K-vectors that are not zero in the first step
+    if (PARTS == 2 && !again) {  // exponents of the K-vectors that are not zero in the first step
       OA.row_max(va[0], rowmax);
       OB.row_max(vb[0], rowmax + 128);
       __syncthreads();
@@ -635,7 +654,7 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
     }
     __syncwarp();
     bool low = false;  // a K-vector that was zero in the first step is badly scaled after it
-    if (open) {
+    if (PARTS == 2 && open) {
       __syncthreads();  // the watched maxima are complete
       if (mine) {
         low = rowmax[tid] != 0u && rowmax[tid] < kWellScaledLo;
