@@ -63,7 +63,7 @@ double direct_us(const DirectPlan& p, int64_t m, int64_t n, int64_t k, int64_t b
   if (scalar) step *= 1.2;
   // Clusters do not fill the GPU's groups of SMs: of 152, clusters of 4, 8 and
   // 16 CTAs reach 144, 120 and 112 (cudaOccupancyMaxActiveClusters).
-  const int size = (p.in_cluster ? p.slices : 1) * (p.pair ? 2 : 1);
+  const int size = direct_cluster_ctas(p);
   double slots = num_sms * (size <= 2 ? 1.0 : size == 4 ? 144.0 / 152 : size == 8 ? 120.0 / 152 : 112.0 / 152);
   if (three && ctas > slots) {  // two CTAs share an SM
     slots *= 2;
@@ -77,9 +77,8 @@ double direct_us(const DirectPlan& p, int64_t m, int64_t n, int64_t k, int64_t b
   return t;
 }
 
-}  // namespace
-
-bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
+// The plan that serves the call best, of clusters of at most max_cluster CTAs.
+bool choose_plan(const SplitCall& c, int num_sms, int max_cluster, DirectPlan* plan, double* us = nullptr) {
   const int64_t m = c.m, n = c.n, k = c.k, batch = c.batch;
   if (c.lda >= (1 << 22) || c.ldb >= (1 << 22)) return false;  // offsets within a tile are 32 bits
   const bool three = split_parts(k) == 2;
@@ -89,7 +88,8 @@ bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
   // 8% in favour of the packed path: over 150 shapes drawn from the ranges of
   // the timed workloads the direct path took 101, was 1.42 times as fast in
   // the mean and never slower.
-  double best = 0.92 * packed_us(m, n, k, batch, num_sms, three);
+  const double packed = packed_us(m, n, k, batch, num_sms, three);
+  double best = 0.92 * packed;
   bool found = false;
   const size_t packed_bytes = split_layout(m, n, k, batch, 1, 256).total;
   auto offer = [&](int bn, bool pair, int64_t slices, bool in_cluster) {
@@ -103,6 +103,7 @@ bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
     }
     DirectPlan p;
     p.bn = bn; p.pair = pair; p.slices = (int)slices; p.in_cluster = in_cluster;
+    if (direct_cluster_ctas(p) > max_cluster) return;
     const int64_t bm = pair ? 256 : 128;
     if ((m + bm - 1) / bm * ((n + bn - 1) / bn) * batch * slices > 0xFFFFFF) return;
     // never more workspace than the packed path's, which callers may have reserved
@@ -121,7 +122,45 @@ bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
     const int64_t tiles = (m + 255) / 256 * ((n + 255) / 256);
     if (batch == 1 && tiles * 4 <= num_sms) offer(256, true, std::min<int64_t>(num_sms / (2 * tiles), 64), false);
   }
+  if (us) us[0] = best, us[1] = packed;
   return found;
+}
+
+}  // namespace
+
+// A cluster that the device cannot place (16 CTAs are beyond the portable
+// size, and a partition of a GPU may have fewer SMs together) gives way to a
+// smaller one, and in the end to the packed path.
+bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan) {
+  const bool three = split_parts(c.k) == 2;
+  const int ma = load_mode(c.ta == 1, c.A, c.lda, c.batch > 1 ? c.sa : 0);
+  const int mb = load_mode(c.tb == 0, c.B, c.ldb, c.batch > 1 ? c.sb : 0);
+  auto fits = three ? (ma == kRows  ? direct_mode_fits<3, kRows>
+                       : ma == kVec ? direct_mode_fits<3, kVec>
+                                    : direct_mode_fits<3, kScalar>)
+                    : (ma == kRows  ? direct_mode_fits<2, kRows>
+                       : ma == kVec ? direct_mode_fits<2, kVec>
+                                    : direct_mode_fits<2, kScalar>);
+  for (int max_cluster = kDirectMaxCluster; max_cluster > 0; max_cluster = direct_cluster_ctas(*plan) / 2) {
+    if (!choose_plan(c, num_sms, max_cluster, plan)) return false;
+    if (fits(*plan, mb)) return true;
+  }
+  return false;
+}
+
+extern "C" int gbgemm_internal_direct_plan(char transa, char transb, int64_t m, int64_t n, int64_t k, int64_t batch,
+                                           int64_t lda, int64_t ldb, int num_sms, int max_cluster, int* plan) {
+  SplitCall c;
+  c.ta = transa != 'N'; c.tb = transb != 'N';
+  c.m = m; c.n = n; c.k = k; c.batch = batch; c.lda = lda; c.ldb = ldb;
+  c.sa = batch > 1 ? lda * (c.ta ? m : k) : 0;
+  c.sb = batch > 1 ? ldb * (c.tb ? k : n) : 0;
+  DirectPlan p;
+  double us[2];
+  if (!choose_plan(c, num_sms, max_cluster, &p, us)) return 0;
+  plan[4] = (int)(1000.0 * us[0]); plan[5] = (int)(1000.0 * us[1]);
+  plan[0] = p.bn; plan[1] = p.pair; plan[2] = p.slices; plan[3] = p.in_cluster;
+  return 1;
 }
 
 cudaError_t launch_direct(const SplitCall& c, const DirectPlan& plan, cudaStream_t s) {
@@ -142,7 +181,7 @@ cudaError_t launch_direct(const SplitCall& c, const DirectPlan& plan, cudaStream
   if ((int64_t)(S.slices - 1) * S.slice_chunks >= S.nkc) return cudaErrorInvalidValue;  // no empty slice
   S.cluster_slices = plan.in_cluster ? plan.slices : 1;
   if (plan.in_cluster && plan.slices > 1 &&
-      (plan.bn % plan.slices || plan.slices * (plan.pair ? 2 : 1) > 16 || plan.bn > 128))
+      (plan.bn % plan.slices || direct_cluster_ctas(plan) > kDirectMaxCluster || plan.bn > 128))
     return cudaErrorInvalidValue;
   S.partial = plan.slices > 1 && !plan.in_cluster ? static_cast<float*>(c.ws) : nullptr;
   if (plan.slices > 1 && !plan.in_cluster && (c.batch != 1 || !c.ws)) return cudaErrorInvalidValue;

@@ -23,7 +23,15 @@ struct DirectArgs {
   int* status;
 };
 
+// CTAs of a plan's clusters.
+inline int direct_cluster_ctas(const DirectPlan& plan) {
+  return (plan.in_cluster ? plan.slices : 1) * (plan.pair ? 2 : 1);
+}
+
 template <int PARTS, int MA>
 cudaError_t launch_direct_mode(const DirectPlan& plan, int mb, const DirectArgs& S, int64_t items, cudaStream_t s);
+// Whether the device can hold a cluster of the plan's instance.
+template <int PARTS, int MA>
+bool direct_mode_fits(const DirectPlan& plan, int mb);
 
 }  // namespace gbg

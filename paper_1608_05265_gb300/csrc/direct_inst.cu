@@ -5,4 +5,5 @@
 namespace gbg {
 template cudaError_t launch_direct_mode<GBG_PARTS, GBG_MODE_A>(const DirectPlan&, int, const DirectArgs&, int64_t,
                                                                cudaStream_t);
+template bool direct_mode_fits<GBG_PARTS, GBG_MODE_A>(const DirectPlan&, int);
 }  // namespace gbg

@@ -61,6 +61,8 @@
 // column first, so that nothing is rounded to a subnormal before the end.
 #pragma once
 
+#include <atomic>
+
 #include "direct.h"
 #include "split_device.cuh"
 
@@ -69,8 +71,6 @@ namespace {
 
 constexpr float kWatchLimit = 0x1p50f;
 constexpr uint64_t kWaitNs = 2000000000ull;
-
-constexpr int kNoExp = -(1 << 20);  // exponent of a K-vector that is zero throughout a slice
 
 // Shape of a kernel instance.  UK k chunks are split per step, each by eight
 // warps of its own.  Two parts: two chunks (16 warps), so that the waits and
@@ -797,56 +797,99 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
   }
 }
 
+// The launch of an instance with clusters of `cluster` CTAs: its attributes
+// are set (once per device), cfg and attr filled in (attr outlives cfg's use).
 template <int BN, bool PAIR, int PARTS, int MA, int MB>
-cudaError_t launch_direct_kernel(const DirectArgs& S, int64_t items, cudaStream_t s) {
+cudaError_t prepare_direct_launch(int dev, int cluster, int64_t ctas, cudaLaunchConfig_t* cfg,
+                                  cudaLaunchAttribute (&attr)[2]) {
   using D = DirectShape<BN, PAIR, PARTS>;
-  static bool attr_set[64] = {};
+  static std::atomic<bool> attr_set[64] = {};
   auto* fn = direct_gemm_kernel<BN, PAIR, PARTS, MA, MB>;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, D::SMEM);
+  if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_relaxed)) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, D::SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(items * (PAIR ? 2 : 1)));
-  cfg.blockDim = dim3(D::THREADS);
-  cfg.dynamicSmemBytes = D::SMEM;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cfg->gridDim = dim3((unsigned)ctas);
+  cfg->blockDim = dim3(D::THREADS);
+  cfg->dynamicSmemBytes = D::SMEM;
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)(S.cluster_slices * (PAIR ? 2 : 1));
+  attr[1].val.clusterDim.x = (unsigned)cluster;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = attr[1].val.clusterDim.x > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, fn, S);
+  cfg->attrs = attr;
+  cfg->numAttrs = cluster > 1 ? 2 : 1;
+  return cudaSuccess;
 }
 
+template <int BN, bool PAIR, int PARTS, int MA, int MB>
+cudaError_t launch_direct_kernel(const DirectArgs& S, int64_t items, cudaStream_t s) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  const int per = PAIR ? 2 : 1;
+  e = prepare_direct_launch<BN, PAIR, PARTS, MA, MB>(dev, S.cluster_slices * per, items * per, &cfg, attr);
+  if (e != cudaSuccess) return e;
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, direct_gemm_kernel<BN, PAIR, PARTS, MA, MB>, S);
+}
+
+// Whether the device can hold a cluster of `cluster` (1, 2, 4, 8, 16) CTAs of
+// an instance, asked once per device.
+template <int BN, bool PAIR, int PARTS, int MA, int MB>
+bool direct_kernel_fits(int cluster) {
+  static std::atomic<signed char> known[64][5] = {};  // 1: fits, -1: does not
+  int dev = 0, bit = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  while (1 << bit < cluster) ++bit;
+  const bool keep = dev >= 0 && dev < 64 && bit < 5;
+  if (keep)
+    if (const signed char k = known[dev][bit].load(std::memory_order_relaxed)) return k > 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  bool fits = prepare_direct_launch<BN, PAIR, PARTS, MA, MB>(dev, cluster, cluster, &cfg, attr) == cudaSuccess;
+  if (fits && cluster > 1) {
+    cfg.attrs = attr + 1;
+    cfg.numAttrs = 1;
+    fits = cudaOccupancyMaxActiveClusters(&n, direct_gemm_kernel<BN, PAIR, PARTS, MA, MB>, &cfg) == cudaSuccess && n > 0;
+  }
+  if (!fits) (void)cudaGetLastError();  // such a cluster is not used: not an error
+  if (keep) known[dev][bit].store(fits ? 1 : -1, std::memory_order_relaxed);
+  return fits;
+}
 
 }  // namespace
 
 // One of the six (parts, mode of op(A)) families of instances, a translation
 // unit each.
+#define GBG_DIRECT_CALL(FN, BN, PAIR, ...)                        \
+  (mb == kRows  ? FN<BN, PAIR, PARTS, MA, kRows>(__VA_ARGS__)      \
+   : mb == kVec ? FN<BN, PAIR, PARTS, MA, kVec>(__VA_ARGS__)       \
+                : FN<BN, PAIR, PARTS, MA, kScalar>(__VA_ARGS__))
 template <int PARTS, int MA>
 cudaError_t launch_direct_mode(const DirectPlan& plan, int mb, const DirectArgs& S, int64_t items, cudaStream_t s) {
-#define GBG_DIRECT_SHAPE(BN, PAIR)                                                      \
-  if (plan.bn == BN && plan.pair == PAIR)                                               \
-    return mb == kRows  ? launch_direct_kernel<BN, PAIR, PARTS, MA, kRows>(S, items, s) \
-           : mb == kVec ? launch_direct_kernel<BN, PAIR, PARTS, MA, kVec>(S, items, s)  \
-                        : launch_direct_kernel<BN, PAIR, PARTS, MA, kScalar>(S, items, s);
-  GBG_DIRECT_SHAPE(64, false)
-  GBG_DIRECT_SHAPE(128, true)
-  if constexpr (PARTS == 2) {
-    GBG_DIRECT_SHAPE(256, true)
-  }
-#undef GBG_DIRECT_SHAPE
+  if (plan.bn == 64 && !plan.pair) return GBG_DIRECT_CALL(launch_direct_kernel, 64, false, S, items, s);
+  if (plan.bn == 128 && plan.pair) return GBG_DIRECT_CALL(launch_direct_kernel, 128, true, S, items, s);
+  if constexpr (PARTS == 2)
+    if (plan.bn == 256 && plan.pair) return GBG_DIRECT_CALL(launch_direct_kernel, 256, true, S, items, s);
   return cudaErrorInvalidValue;
 }
+
+template <int PARTS, int MA>
+bool direct_mode_fits(const DirectPlan& plan, int mb) {
+  const int cluster = direct_cluster_ctas(plan);
+  if (plan.bn == 64 && !plan.pair) return GBG_DIRECT_CALL(direct_kernel_fits, 64, false, cluster);
+  if (plan.bn == 128 && plan.pair) return GBG_DIRECT_CALL(direct_kernel_fits, 128, true, cluster);
+  if constexpr (PARTS == 2)
+    if (plan.bn == 256 && plan.pair) return GBG_DIRECT_CALL(direct_kernel_fits, 256, true, cluster);
+  return false;
+}
+#undef GBG_DIRECT_CALL
 
 }  // namespace gbg

@@ -150,21 +150,31 @@ struct SplitCall {
 // reduction).
 cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s);
 
-// A split-path call without a packing pass (direct.cu): tiles of 128 x bn (bn
-// 64 or 128) or, pair, of 256 x bn (128 or 256), k in `slices` ranges, summed
-// in the cluster (bn a multiple of slices and at most 128, at most 16 CTAs) or
-// through c.ws (slices x the output's tiles raw 128 x bn accumulators).
-// Exponents of one slice's tile: whether any is set, those of its 128 rows and
-// (at most 256) columns.
+// Exponents of one slice's tile on the direct path: whether any is set, those
+// of its 128 rows and (at most 256) columns; kNoExp for a K-vector that is
+// zero throughout the slice.
 constexpr int kDirectExpInts = 1 + 128 + 256;
+constexpr int kNoExp = -(1 << 20);
+constexpr int kDirectMaxCluster = 16;  // CTAs
+// A split-path call without a packing pass (direct.cu): tiles of 128 x 64 or,
+// pair, of 256 x 128 or 256 x 256, k in `slices` ranges, summed in the cluster
+// (bn a multiple of slices and at most 128, at most kDirectMaxCluster CTAs) or
+// through c.ws (slices x the output's tiles raw 128 x bn accumulators).
 struct DirectPlan {
-  int bn = 128;
+  int bn = 64;
   bool pair = false;
   int slices = 1;
   bool in_cluster = true;
 };
-// Whether the direct path serves a call better than the packed one, and how.
+// Whether the direct path serves a call better than the packed one, and how,
+// with clusters that the current device can place.
 bool direct_plan(const SplitCall& c, int num_sms, DirectPlan* plan);
+// The rule alone, for tests (no GPU; aligned operands at the given leading
+// dimensions, clusters of at most max_cluster CTAs): 1 and plan[0 .. 5] = bn,
+// pair, slices, in_cluster, the estimated times of this plan and of the packed
+// path in ns; or 0 where the packed path serves the call.
+extern "C" int gbgemm_internal_direct_plan(char transa, char transb, int64_t m, int64_t n, int64_t k, int64_t batch,
+                                           int64_t lda, int64_t ldb, int num_sms, int max_cluster, int* plan);
 size_t direct_workspace_bytes(int64_t m, int64_t n, const DirectPlan& plan);
 cudaError_t launch_direct(const SplitCall& c, const DirectPlan& plan, cudaStream_t s);
 

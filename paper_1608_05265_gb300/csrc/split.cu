@@ -40,10 +40,9 @@ namespace {
 // throughout has kNoExp there and adds nothing).
 __device__ __noinline__ float4 rescaled_sum(const float4* p, size_t slice_elems, int splitk, const int* pexp,
                                             size_t pstride, int row, int col) {
-  constexpr int kNone = -(1 << 19);
   float out[4];
   for (int q = 0; q < 4; ++q) {
-    int er = 2 * kNone, ec = 2 * kNone;
+    int er = kNoExp, ec = kNoExp;
     for (int s = 0; s < splitk; ++s) {
       er = max(er, pexp[s * pstride + 1 + row + q]);
       ec = max(ec, pexp[s * pstride + 129 + col]);
