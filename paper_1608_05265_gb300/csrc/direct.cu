@@ -24,12 +24,13 @@ size_t direct_workspace_bytes(int64_t m, int64_t n, const DirectPlan& plan) {
 namespace {
 
 // Estimated time (us) of a call on the packed path, as its launch chooses
-// tiles, pairs and k slices (split.cu, default_schedule): the launches, the
-// packing at its measured 4.8 TB/s, rounds of tiles at the measured time per
-// 32-deep chunk, the accumulators' way out, and the split-K reduction.
-// Against measurements at 256^3 .. 4096^3, ragged, tall, batched and long-k
-// shapes: within 15%, and up to 2.5 us too much since the packing is launched
-// ahead of the clearing (no shape drawn since was slower for it, see below).
+// tiles, pairs and k slices (split.cu, default_schedule): the launches and the
+// packing, rounds of tiles at a time per 32-deep chunk, the accumulators' way
+// out, and the split-K reduction.  The constants here and in direct_us are
+// fitted to measured calls, three sets of operands in turn (m, n log-uniform
+// in 64 .. 6000, k in 128 .. 65536, batches to 96): this to 1000 calls, within
+// 10% of nearly all, up to 40% too little where pair tiles wait for packed
+// panels (k just above 512); that to 3384 plans of 450 calls.
 double packed_us(int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bool three) {
   const double nkc = (double)panel_k_chunks(k);
   const int64_t tm = (m + 127) / 128;
@@ -37,43 +38,49 @@ double packed_us(int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bo
   int bn = tiles(256) >= num_sms / 2 ? 256 : tiles(128) >= num_sms / 2 ? 128 : 64;
   int s = batch == 1 ? choose_splitk((int64_t)tiles(256), k, num_sms) : 1;
   if (s > 1) bn = 256;
-  double t = 12.5 + (three ? 10.0 : 8.0) * (double)k * (double)(m + n) * (double)batch / 4.8e6;
-  if (s > 1) t += 5.0;
+  double t = 11.6 + (three ? 2.33e-6 : 1.87e-6) * (double)k * (double)(m + n) * (double)batch;
+  if (s > 1) t += 3.5;
   const double chunks = std::ceil(nkc / s);
   if (bn == 256 && tm >= 2 && (!three || nkc >= 8)) {
     if (s == 1) return t + choose_pair_tiles(m, n, batch, panel_k_chunks(k), three, num_sms / 2).us;
     const double items = (double)((tm + 1) / 2 * ((n + 255) / 256) * batch) * s;
     return t + std::ceil(items / (num_sms / 2)) * (chunks * (three ? 1.0 : 0.5) + 4.0);
   }
-  const double per = bn == 256 ? 0.55 : bn == 128 ? 0.42 : 0.4;
-  return t + std::ceil(tiles(bn) * s / num_sms) * (chunks * per * (three ? 1.8 : 1.0) + 2.0);
+  const double per = bn == 256 ? 0.6 : bn == 128 ? 0.44 : 0.37;
+  return t + std::ceil(tiles(bn) * s / num_sms) * (chunks * per * (three ? 1.8 : 1.0) + 1.5);
 }
 
-// The same for a plan of the direct path.  Per 64-deep step 1.30 / 1.33 /
-// 1.58 us of a 64 / 128 / 256 wide tile (from 512 x 512 x 65536 without
-// slices), per 32-deep step with three parts 0.8 / 1.05; 1.2 times that with
-// operands whose rows are not 16-byte aligned.
+// The same for a plan of the direct path.  Two parts: per 64-deep step 1.25 /
+// 1.36 / 1.61 us of a 64 / 128 / 256 wide tile; three parts: per 32-deep step
+// 1.0 / 1.32, and 1.63 times that for two CTAs on an SM.  1.2 times that with
+// one operand whose rows are not 16-byte aligned, 1.3 with two.  The sum of
+// slices in a cluster goes by rounds of four columns a thread.  A CTA serves
+// one tile: every further round of CTAs starts anew.  Of the 450 calls, the
+// plan this and packed_us choose takes 1.008 times the best one's time in the
+// geometric mean, at most 1.29, and at most 1.02 of the packed path's.
 double direct_us(const DirectPlan& p, int64_t m, int64_t n, int64_t k, int64_t batch, int num_sms, bool three,
-                 bool scalar) {
+                 int scalars) {
   const int bm = p.pair ? 256 : 128;
   const double ctas = (double)((m + bm - 1) / bm * ((n + p.bn - 1) / p.bn) * batch) * p.slices * (p.pair ? 2 : 1);
   const double chunks = std::ceil((double)panel_k_chunks(k) / p.slices);
   const double steps = three ? chunks : std::ceil(chunks / 2);
-  double step = three ? (p.bn == 64 ? 0.8 : 1.05) : p.bn == 64 ? 1.30 : p.bn == 128 ? 1.33 : 1.58;
-  if (scalar) step *= 1.2;
+  double step = three ? (p.bn == 64 ? 1.0 : 1.32) : p.bn == 64 ? 1.25 : p.bn == 128 ? 1.36 : 1.61;
+  step *= scalars == 2 ? (three ? 1.3 : 1.35) : scalars == 1 ? 1.2 : 1.0;
   // Clusters do not fill the GPU's groups of SMs: of 152, clusters of 4, 8 and
-  // 16 CTAs reach 144, 120 and 112 (cudaOccupancyMaxActiveClusters).
+  // 16 CTAs reach 144, 120 and 112 (cudaOccupancyMaxActiveClusters on GB300).
   const int size = direct_cluster_ctas(p);
   double slots = num_sms * (size <= 2 ? 1.0 : size == 4 ? 144.0 / 152 : size == 8 ? 120.0 / 152 : 112.0 / 152);
+  double again = three ? 3.0 : 5.8;
   if (three && ctas > slots) {  // two CTAs share an SM
     slots *= 2;
-    step *= 2.2;
+    step *= 1.63;
+    again = 4.0;
   }
   const double waves = std::ceil(ctas / slots);
-  const double out = p.bn * 0.03;  // a tile's way out: not hidden behind the next one
-  double t = (p.pair ? 9.0 : p.slices > 1 ? 6.5 : 4.5) + waves * (steps * step + out);
-  if (p.slices > 1 && p.pair) t += 2.5;
-  if (p.slices > 1 && !p.in_cluster) t += 4.0;
+  const double out = three ? 0.0 : p.bn * 0.018;  // a tile's way out: not hidden behind the next one
+  double t = (three ? 6.7 : 5.2) + waves * (steps * step + out) + (waves - 1) * again;
+  if (p.slices > 1)
+    t += !p.in_cluster ? 7.0 : three ? 0.9 * ((p.bn / p.slices + 7) / 8) + 0.2 * p.slices : 1.15 * ((p.bn / p.slices + 15) / 16);
   return t;
 }
 
@@ -83,13 +90,13 @@ bool choose_plan(const SplitCall& c, int num_sms, int max_cluster, DirectPlan* p
   if (c.lda >= (1 << 22) || c.ldb >= (1 << 22)) return false;  // offsets within a tile are 32 bits
   const bool three = split_parts(k) == 2;
   const int64_t nkc = panel_k_chunks(k);
-  const bool scalar = load_mode(c.ta == 1, c.A, c.lda, batch > 1 ? c.sa : 0) == kScalar ||
-                      load_mode(c.tb == 0, c.B, c.ldb, batch > 1 ? c.sb : 0) == kScalar;
-  // 8% in favour of the packed path: over 150 shapes drawn from the ranges of
-  // the timed workloads the direct path took 101, was 1.42 times as fast in
-  // the mean and never slower.
+  const int scalars = (load_mode(c.ta == 1, c.A, c.lda, batch > 1 ? c.sa : 0) == kScalar) +
+                      (load_mode(c.tb == 0, c.B, c.ldb, batch > 1 ? c.sb : 0) == kScalar);
+  // In favour of the packed path, for the estimates' error.  Over 500 further
+  // calls drawn alike, path AUTO then takes 0.745 times the packed path's time
+  // in the geometric mean and at most 1.01 times (with 4% both ways up to 1.09).
   const double packed = packed_us(m, n, k, batch, num_sms, three);
-  double best = 0.92 * packed;
+  double best = (three ? 0.9 : 0.94) * packed;
   bool found = false;
   const size_t packed_bytes = split_layout(m, n, k, batch, 1, 256).total;
   auto offer = [&](int bn, bool pair, int64_t slices, bool in_cluster) {
@@ -108,7 +115,7 @@ bool choose_plan(const SplitCall& c, int num_sms, int max_cluster, DirectPlan* p
     if ((m + bm - 1) / bm * ((n + bn - 1) / bn) * batch * slices > 0xFFFFFF) return;
     // never more workspace than the packed path's, which callers may have reserved
     if (direct_workspace_bytes(m, n, p) > packed_bytes) return;
-    const double t = direct_us(p, m, n, k, batch, num_sms, three, scalar);
+    const double t = direct_us(p, m, n, k, batch, num_sms, three, scalars);
     if (t < best) {
       best = t;
       *plan = p;
