@@ -28,7 +28,7 @@ HEADERS = [os.path.join(CSRC, h) for h in ("internal.h", "split_device.cuh", "si
                                             "grouped.h", "tuner.h", "mlp.h", "direct.h", "direct_kernel.cuh")] + \
     [os.path.join(ROOT, "include", "gbgemm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "-Xptxas", "-v",
          "-I" + os.path.join(ROOT, "include")]
 
 
@@ -61,6 +61,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")
+        with open(os.path.join(OUT, name + ".ptxas"), "w") as f:  # registers, spills and shared memory of every kernel
+            f.write(r.stderr)
         if verbose:
             sys.stderr.write(r.stderr)
         return obj

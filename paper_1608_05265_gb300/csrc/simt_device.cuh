@@ -155,8 +155,10 @@ struct SliceLoader {
 
 // One BM x BN tile of C = alpha*op(A)*op(B) + beta*C starting at (m0, n0),
 // computed by the (BM/8)*(BN/8) threads of the calling block.  As and Bs are
-// the block's two-buffer shared-memory slices (SimtSmem<BM, BN>).
-template <int BM, int BN, bool TA, bool TB, bool VEC>
+// the block's two-buffer shared-memory slices (SimtSmem<BM, BN>).  JB: the
+// columns of C that the epilogue loads before it stores any, 0 for four rows
+// of one column at a time.
+template <int BM, int BN, bool TA, bool TB, bool VEC, int JB>
 __device__ __forceinline__ void simt_tile(const Problem& P, int64_t m0, int64_t n0,
                                           float (*As)[BK * (BM + 4)], float (*Bs)[BK * (BN + 4)]) {
   using T = SimtTile<BM, BN, TA, TB, VEC>;
@@ -235,85 +237,82 @@ __device__ __forceinline__ void simt_tile(const Problem& P, int64_t m0, int64_t 
   // rounding of beta*c and one of the sum (fmaf), so that k = 1 stays within
   // 2*2^-24 of the exact value.  The C of JB columns is loaded before any of
   // it is stored: one by one, each load waited for the store before it (the
-  // compiler cannot tell them apart; 4608^2 with k = 32: 84 -> 52 us).  The
-  // widest tile of two transposed operands keeps one column at a time (its
-  // multiply loop came out 15% slower with more: 4096^3 TT 3126 -> 3600 us).
+  // compiler cannot tell them apart; 4608^2 with k = 32: 84 -> 52 us).
   const bool vec_c = ((P.ldc & 3) == 0) && ((reinterpret_cast<uintptr_t>(P.C) & 15) == 0);
-  if constexpr (VEC && TA && TB && BM == 128 && BN == 128) {
+  if constexpr (JB == 0) {
 #pragma unroll
-  for (int jh = 0; jh < 2; ++jh) {
+    for (int jh = 0; jh < 2; ++jh) {
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int64_t j = n0 + jh * (BN / 2) + tx * 4 + jj;
-      if (j >= P.n) continue;
+      for (int jj = 0; jj < 4; ++jj) {
+        const int64_t j = n0 + jh * (BN / 2) + tx * 4 + jj;
+        if (j >= P.n) continue;
 #pragma unroll
-      for (int ih = 0; ih < 2; ++ih) {
-        const int64_t i = m0 + ih * (BM / 2) + ty * 4;
-        float* cp = P.C + i + j * P.ldc;
-        float v[4];
+        for (int ih = 0; ih < 2; ++ih) {
+          const int64_t i = m0 + ih * (BM / 2) + ty * 4;
+          float* cp = P.C + i + j * P.ldc;
+          float v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = acc[ih * 4 + q][jh * 4 + jj];
-        if (vec_c && i + 3 < P.m) {
-          if (P.beta != 0.f) {
-            const float4 c = *reinterpret_cast<const float4*>(cp);
-            v[0] = fmaf(P.alpha, v[0], P.beta * c.x); v[1] = fmaf(P.alpha, v[1], P.beta * c.y);
-            v[2] = fmaf(P.alpha, v[2], P.beta * c.z); v[3] = fmaf(P.alpha, v[3], P.beta * c.w);
+          for (int q = 0; q < 4; ++q) v[q] = acc[ih * 4 + q][jh * 4 + jj];
+          if (vec_c && i + 3 < P.m) {
+            if (P.beta != 0.f) {
+              const float4 c = *reinterpret_cast<const float4*>(cp);
+              v[0] = fmaf(P.alpha, v[0], P.beta * c.x); v[1] = fmaf(P.alpha, v[1], P.beta * c.y);
+              v[2] = fmaf(P.alpha, v[2], P.beta * c.z); v[3] = fmaf(P.alpha, v[3], P.beta * c.w);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) v[q] = P.alpha * v[q];
+            }
+            *reinterpret_cast<float4*>(cp) = make_float4(v[0], v[1], v[2], v[3]);
           } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = P.alpha * v[q];
-          }
-          *reinterpret_cast<float4*>(cp) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (i + q < P.m) cp[q] = (P.beta != 0.f) ? fmaf(P.alpha, v[q], P.beta * cp[q]) : P.alpha * v[q];
+            for (int q = 0; q < 4; ++q) {
+              if (i + q < P.m) cp[q] = (P.beta != 0.f) ? fmaf(P.alpha, v[q], P.beta * cp[q]) : P.alpha * v[q];
+            }
           }
         }
       }
     }
-  }
-    return;
-  }
-  constexpr int JB = 4;
+  } else {
 #pragma unroll
-  for (int jb = 0; jb < 8; jb += JB) {
-    const int64_t j0 = n0 + (jb >> 2) * (BN / 2) + tx * 4 + (jb & 3);
-    float c[JB][2][4];
-    if (P.beta != 0.f) {
+    for (int jb = 0; jb < 8; jb += JB) {
+      const int64_t j0 = n0 + (jb >> 2) * (BN / 2) + tx * 4 + (jb & 3);
+      float c[JB][2][4];
+      if (P.beta != 0.f) {
 #pragma unroll
-      for (int jj = 0; jj < JB; ++jj)
+        for (int jj = 0; jj < JB; ++jj)
+#pragma unroll
+          for (int ih = 0; ih < 2; ++ih) {
+            const int64_t i = m0 + ih * (BM / 2) + ty * 4;
+            const float* cp = P.C + i + (j0 + jj) * P.ldc;
+            if (j0 + jj < P.n && vec_c && i + 3 < P.m) {
+              const float4 f = *reinterpret_cast<const float4*>(cp);
+              c[jj][ih][0] = f.x; c[jj][ih][1] = f.y; c[jj][ih][2] = f.z; c[jj][ih][3] = f.w;
+            } else {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) c[jj][ih][q] = (j0 + jj < P.n && i + q < P.m) ? cp[q] : 0.f;
+            }
+          }
+      }
+#pragma unroll
+      for (int jj = 0; jj < JB; ++jj) {
+        if (j0 + jj >= P.n) continue;
 #pragma unroll
         for (int ih = 0; ih < 2; ++ih) {
           const int64_t i = m0 + ih * (BM / 2) + ty * 4;
-          const float* cp = P.C + i + (j0 + jj) * P.ldc;
-          if (j0 + jj < P.n && vec_c && i + 3 < P.m) {
-            const float4 f = *reinterpret_cast<const float4*>(cp);
-            c[jj][ih][0] = f.x; c[jj][ih][1] = f.y; c[jj][ih][2] = f.z; c[jj][ih][3] = f.w;
+          float* cp = P.C + i + (j0 + jj) * P.ldc;
+          float v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float a = acc[ih * 4 + q][jb + jj];
+            v[q] = P.beta != 0.f ? fmaf(P.alpha, a, P.beta * c[jj][ih][q]) : P.alpha * a;
+          }
+          if (vec_c && i + 3 < P.m) {
+            *reinterpret_cast<float4*>(cp) = make_float4(v[0], v[1], v[2], v[3]);
           } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) c[jj][ih][q] = (j0 + jj < P.n && i + q < P.m) ? cp[q] : 0.f;
+            for (int q = 0; q < 4; ++q)
+              if (i + q < P.m) cp[q] = v[q];
           }
-        }
-    }
-#pragma unroll
-    for (int jj = 0; jj < JB; ++jj) {
-      if (j0 + jj >= P.n) continue;
-#pragma unroll
-      for (int ih = 0; ih < 2; ++ih) {
-        const int64_t i = m0 + ih * (BM / 2) + ty * 4;
-        float* cp = P.C + i + (j0 + jj) * P.ldc;
-        float v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float a = acc[ih * 4 + q][jb + jj];
-          v[q] = P.beta != 0.f ? fmaf(P.alpha, a, P.beta * c[jj][ih][q]) : P.alpha * a;
-        }
-        if (vec_c && i + 3 < P.m) {
-          *reinterpret_cast<float4*>(cp) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (i + q < P.m) cp[q] = v[q];
         }
       }
     }

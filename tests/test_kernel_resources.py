@@ -1,0 +1,22 @@
+"""What the compiler says of the kernels: the grouped SIMT kernels keep their
+sums in registers (some bytes beside the loop are fine, hundreds are not)."""
+
+import os
+import re
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def info():
+    from paper_1608_05265_gb300 import build
+    build.build()
+    path = os.path.join(build.OUT, "grouped.ptxas")
+    return open(path).read()
+
+
+def test_grouped_simt_kernels_do_not_spill(info):
+    found = re.findall(r"Compiling entry function '(\w*grouped_simt_kernel\w*)'.*?(\d+) bytes spill stores, "
+                       r"(\d+) bytes spill loads", info, re.S)
+    assert len(found) == 24
+    assert max(int(stores) for _, stores, _ in found) <= 100, found
