@@ -126,14 +126,13 @@ __global__ void __launch_bounds__(kGemvNThreads, 2) gemv_n_kernel(int64_t m, int
 
 // Partial (or final) y_j for columns j .. j+3 over rows [i0, i1) (i0 a
 // multiple of 4).  V = 4 (columns that start on 16 bytes): four rows a thread
-// and load, two loads of each column in flight; V = 1: four loads of 4 bytes
-// of each column in flight.
+// and load, U = 2 loads of each column in flight; V = 1: U = 4 (or 2, with more
+// blocks on an SM) loads of 4 bytes of each column in flight.
 template <int V, int U>
-__global__ void __launch_bounds__(kGemvThreads, V == 4 ? 3 : U == 4 ? 4 : 6) gemv_t_kernel(int64_t m, int64_t n, const float* __restrict__ A,
-                                                                 int64_t lda, const float* __restrict__ x,
-                                                                 int64_t incx, int64_t slice,
-                                                                 float* __restrict__ partial, float alpha, float beta,
-                                                                 float* __restrict__ y, int64_t incy) {
+__global__ void __launch_bounds__(kGemvThreads, V == 4 ? 3 : U == 4 ? 4 : 6)
+    gemv_t_kernel(int64_t m, int64_t n, const float* __restrict__ A, int64_t lda, const float* __restrict__ x,
+                  int64_t incx, int64_t slice, float* __restrict__ partial, float alpha, float beta,
+                  float* __restrict__ y, int64_t incy) {
   constexpr int ACC = V == 4 ? 4 : 2;    // sums per column
   __shared__ float red[kTCols][kGemvThreads / 32];
   const int64_t jb = (int64_t)blockIdx.x * kTCols;
@@ -152,10 +151,10 @@ __global__ void __launch_bounds__(kGemvThreads, V == 4 ? 3 : U == 4 ? 4 : 6) gem
   int64_t i = i0 + V * threadIdx.x;
   for (; i < i1; i += U * step) {
     float w[U][kTCols][V], xv[U][V];
-    const bool full = i + (U - 1) * step + V <= i1;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t r = i + u * step;
+      const bool full = r + V <= i1;  // by step: of the last rows most threads still have four
 #pragma unroll
       for (int c = 0; c < kTCols; ++c) {
         if (V == 4 && full) {
@@ -302,9 +301,17 @@ cudaError_t launch_gemv(bool trans, int64_t m, int64_t n, float alpha, const flo
     const int64_t slice = ceil_div(ceil_div(m, slices), 4) * 4;
     const dim3 grid((unsigned)ceil_div(n, kTCols), (unsigned)ceil_div(m, slice));
     if (ceil_div(n, kTCols) > 0x7FFFFFFF) return cudaErrorInvalidConfiguration;
-    // fewer than 1024 rows are one step of every thread: as many blocks on an
-    // SM as can be (300 x 12000: 8.4 us, with four rows a thread 9.6)
-    auto kernel = slice < 1024 ? gemv_t_kernel<1, 2> : vec ? gemv_t_kernel<4, 2> : gemv_t_kernel<1, 4>;
+    // Few rows are a few steps of every thread: as many blocks on an SM as can
+    // be (aligned, four rows a thread in <4, 2>: 300 x 12000 9.6 against 8.4
+    // us, 1025 x 4096 8.4 against 7.2, 1100 x 16384 24.8 against 20.8), and so
+    // for unaligned columns whose blocks would come in a second round (16384 x
+    // 2500, ld + 1: 39 against 35).
+    const int64_t blocks = (int64_t)grid.x * grid.y;
+    const bool second = slice > 4096 && blocks > 4 * num_sms && blocks <= 6 * num_sms;
+    auto kernel = slice <= 2304 ? gemv_t_kernel<1, 2>
+                  : vec         ? gemv_t_kernel<4, 2>
+                  : second      ? gemv_t_kernel<1, 2>
+                                : gemv_t_kernel<1, 4>;
     kernel<<<grid, kGemvThreads, 0, s>>>(m, n, A, lda, x, incx, slice, part, alpha, beta, y, incy);
     slices = grid.y;
   }
