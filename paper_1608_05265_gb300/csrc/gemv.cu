@@ -301,17 +301,17 @@ cudaError_t launch_gemv(bool trans, int64_t m, int64_t n, float alpha, const flo
     const int64_t slice = ceil_div(ceil_div(m, slices), 4) * 4;
     const dim3 grid((unsigned)ceil_div(n, kTCols), (unsigned)ceil_div(m, slice));
     if (ceil_div(n, kTCols) > 0x7FFFFFFF) return cudaErrorInvalidConfiguration;
-    // Few rows are a few steps of every thread: as many blocks on an SM as can
-    // be (aligned, four rows a thread in <4, 2>: 300 x 12000 9.6 against 8.4
-    // us, 1025 x 4096 8.4 against 7.2, 1100 x 16384 24.8 against 20.8), and so
-    // for unaligned columns whose blocks would come in a second round (16384 x
-    // 2500, ld + 1: 39 against 35).
+    // Four rows a thread from 4096 on (16384^2 148 against 164 us): below, their
+    // steps are few and long (1025 x 4096: 8.5 against 6.5 us, 1500 x 16384 29.4
+    // against 26.5).  Two loads of 4 bytes in flight, but more blocks on an SM,
+    // below 1024 rows, where a step is all (300 x 12000: 8.4 us, four rows a
+    // thread 9.6), below 2048 with many rounds of blocks (1500 x 16384: 23.3),
+    // and where a second round would be nearly empty (4097 x 2500, ld + 1: 12.5
+    // against 14.5).
     const int64_t blocks = (int64_t)grid.x * grid.y;
-    const bool second = slice > 4096 && blocks > 4 * num_sms && blocks <= 6 * num_sms;
-    auto kernel = slice <= 2304 ? gemv_t_kernel<1, 2>
-                  : vec         ? gemv_t_kernel<4, 2>
-                  : second      ? gemv_t_kernel<1, 2>
-                                : gemv_t_kernel<1, 4>;
+    const bool two = slice < 1024 || (slice < 2048 && blocks > 16 * num_sms) ||
+                     (!vec && slice > 4096 && blocks > 4 * num_sms && blocks <= 6 * num_sms);
+    auto kernel = two ? gemv_t_kernel<1, 2> : vec && slice > 4096 ? gemv_t_kernel<4, 2> : gemv_t_kernel<1, 4>;
     kernel<<<grid, kGemvThreads, 0, s>>>(m, n, A, lda, x, incx, slice, part, alpha, beta, y, incy);
     slices = grid.y;
   }
