@@ -86,6 +86,12 @@ __global__ void __launch_bounds__(kGemvNThreads, 2) gemv_n_kernel(int64_t m, int
             for (int v = 0; v < 4; ++v) w[u][v] = __ldg(col + u * lda + v * VS);
           }
         }
+      } else if (VEC && rows == 4) {  // the last columns
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float4 f = u < cnt ? __ldg(reinterpret_cast<const float4*>(col + u * lda)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          w[u][0] = f.x; w[u][1] = f.y; w[u][2] = f.z; w[u][3] = f.w;
+        }
       } else {  // the last columns, or the last rows
 #pragma unroll
         for (int u = 0; u < U; ++u)
@@ -289,8 +295,10 @@ cudaError_t launch_gemv(bool trans, int64_t m, int64_t n, float alpha, const flo
     // Rows per block (4 rt): with aligned columns as many as can be, for the
     // memory's sake (16384^2, from cold: 1024 rows 173 us, 512 rows 197, one
     // row a thread 195); with others 256 (ld + 1: 185 us, 512 rows 201, one row
-    // a thread 193); 512 for the few rows of a short y, 256 below.
-    const int rt = m <= 256 ? 64 : m <= 1024 ? 128 : vec ? 256 : 64;
+    // a thread 193); 512 for the few rows of a short y, 256 below; 512 where a
+    // slice has too few columns for two shares (16384 x 20: 4.6 us, with 1024
+    // rows 6.0).
+    const int rt = m <= 256 ? 64 : m <= 1024 ? 128 : vec ? (slice <= 64 ? 128 : 256) : 64;
     const dim3 grid((unsigned)ceil_div(m, 4 * rt), (unsigned)ceil_div(n, slice));
     if (ceil_div(m, 4 * rt) > 0x7FFFFFFF) return cudaErrorInvalidConfiguration;
     auto kernel = vec ? (rt == 64 ? gemv_n_kernel<true, 64> : rt == 128 ? gemv_n_kernel<true, 128> : gemv_n_kernel<true, 256>)

@@ -74,3 +74,16 @@ def test_transposed_time_does_not_jump(h):
     """One row more than a step of four rows a thread cost 1.56 times the time."""
     assert timed(h, "T", 1100, 16384, 0) <= 1.3 * timed(h, "T", 1000, 16384, 0)
     assert timed(h, "T", 1025, 4096, 0) <= 1.2 * timed(h, "T", 1025, 4096, 1)
+
+
+@pytest.mark.parametrize("pad", [0, 1])
+@pytest.mark.parametrize("m,n", [(1025, 1), (1030, 20), (1536, 9), (2050, 64), (3000, 65), (5003, 3), (16384, 20)])
+def test_not_transposed_few_columns(h, m, n, pad):
+    check(h, "N", m, n, pad)
+    check(h, "N", m, n, pad, incx=-3)
+
+
+def test_few_columns_cost_no_more_aligned_than_not(h):
+    """Blocks of 1024 rows took 1.3 times as long as those of unaligned columns."""
+    assert timed(h, "N", 16384, 20, 0) <= 1.15 * timed(h, "N", 16384, 20, 1)
+    assert timed(h, "N", 4097, 20, 0) <= 1.15 * timed(h, "N", 4097, 20, 1)
