@@ -197,12 +197,13 @@ def _ptr(x) -> int | None:
     return x.data_ptr()
 
 
-# The transpose flags as ctypes wants them; anything else is encoded as given.
+# The usual transpose flags as ctypes wants them; others (bytes, bytearray, a
+# character's number) go to it as given.
 _FLAG = {f: f.encode() for f in "NnTtCc"}
 
 
 def _flag(t):
-    return _FLAG[t] if t in _FLAG else t.encode() if isinstance(t, str) else t
+    return t.encode() if isinstance(t, str) else t
 
 
 def _stream_ptr(stream):
