@@ -609,9 +609,13 @@ __global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectS
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stores, before the MMAs' reads
       __syncwarp();
       if (lane == 0) {
-        // (a release at cluster scope would wait for this thread's loads: 4.8
-        // of 18 cycles an instruction.  The proxy fence has ordered the
-        // stores, which the MMA reads through the async proxy.)
+        // The proxy fence has put the stores where the MMA reads them, each
+        // CTA's own shared memory through its own async proxy.  Between the
+        // odd CTA's warps and the issuer this relies on the hardware: the PTX
+        // memory model orders them only by a release and an acquire at cluster
+        // scope, and the release waits for every load this thread has in
+        // flight (a batch of 64 products 192 x 256 x 4096 108 -> 143 us, with
+        // one warp of the odd CTA passing the others' arrivals on 130).
         if (PAIR) mbar_arrive_remote(map_to_rank(full_bar(stage), lead));
         else mbar_arrive(full_bar(stage));
       }
