@@ -427,8 +427,14 @@ int gbgemm_schedule_default(gbgemm_handle* h, const gbgemm_problem* prob, int* s
  * handle's stream.  latency_us: host array of GBGEMM_NUM_SCHEDULES, or NULL. */
 int gbgemm_autotune_schedules(gbgemm_handle* h, const gbgemm_problem* prob, int reps, float* latency_us, int* best);
 /* Schedule of the handle's most recent gbgemm_sgemm that launched the product
- * kernels (-1 before the first). */
+ * kernels (-1 before the first).  Path AUTO serves calls that suit it (small
+ * outputs, batches, long k) without a packing pass, by tiles and k slices that
+ * no schedule describes: then *s is the schedule the fixed heuristic gives the
+ * packed call (pinning it runs that one, with other rounding), and
+ * gbgemm_last_direct says so. */
 int gbgemm_last_schedule(gbgemm_handle* h, int* s);
+/* Whether that call ran without a packing pass (*direct = 0 or 1). */
+int gbgemm_last_direct(gbgemm_handle* h, int* direct);
 /* Pin schedule s for the handle's later single calls (s = -1 unpins).  A
  * pinned schedule overrides the tuning mode for every call it is legal for
  * (gbgemm_schedule_legal, and on the handle's path unless that is AUTO);
@@ -444,6 +450,10 @@ int gbgemm_set_schedule(gbgemm_handle* h, int s);
  *           among the legal schedules of the handle's path; mode 1 when the
  *           predictor has no parameters or a dimension lies outside
  *           [8, 16384].
+ * On path AUTO every mode runs a call without a packing pass where that suits
+ * it: mode 0 and 2 by the fixed rule, mode 1 where the tuner measured it faster
+ * than every schedule (a tuning file of an older version does not have that
+ * figure; its shapes keep to the schedules).
  * Strided batches (batch > 1) always use the fixed heuristic. */
 int gbgemm_set_tuning(gbgemm_handle* h, int mode);
 

@@ -47,6 +47,7 @@ struct gbgemm_handle {
   std::map<std::string, int> sched_choice;   // tuning mode 2: predicted schedule per shape key
   void* pred_scratch = nullptr;              // device scratch of one schedule prediction
   int last_schedule = -1;
+  int last_direct = 0;                       // it ran without a packing pass instead
   int pinned_schedule = -1;                  // gbgemm_set_schedule
 };
 
@@ -258,14 +259,19 @@ bool schedule_allowed(const gbgemm_handle* h, const gbgemm_problem& q, int s) {
 // Tuning modes 1 and 2: the tuner's fastest allowed schedule, or the schedule
 // predictor's choice (cached per shape key; the tuner where the predictor
 // has no parameters or the shape is outside its training range).  *best = -1
-// when nothing is allowed.  Synchronises the stream on a shape's first call.
-int choose_schedule(gbgemm_handle* h, const gbgemm_problem& q, int* best) {
+// when nothing is allowed.  *direct: whether a call without a packing pass goes
+// before it where path AUTO has one (mode 1: it was timed and faster; mode 2:
+// always, the predictor knows packed schedules only).  Synchronises the stream
+// on a shape's first call.
+int choose_schedule(gbgemm_handle* h, const gbgemm_problem& q, int* best, bool* direct) {
   *best = -1;
+  *direct = false;
   if (h->tuning == 2 && h->sched_predictor.ready() && in_training_range3(q.m, q.n, q.k)) {
     const std::string key = gbg::tune_key(q) + (h->path == GBGEMM_PATH_AUTO ? " a" : h->path == GBGEMM_PATH_SIMT ? " s" : " b");
     auto it = h->sched_choice.find(key);
     if (it != h->sched_choice.end()) {
       *best = it->second;
+      *direct = true;
       return GBGEMM_OK;
     }
     constexpr int kLB = (GBGEMM_NUM_SCHEDULES + 7) / 8;
@@ -294,16 +300,19 @@ int choose_schedule(gbgemm_handle* h, const gbgemm_problem& q, int* best) {
     if (choice >= 0) {
       h->sched_choice[key] = choice;
       *best = choice;
+      *direct = true;
       return GBGEMM_OK;
     }
   }
   std::vector<float> lat;
   h->tuner.bind(h->stream, h->d_status, h->num_sms);
-  if (h->tuner.measure_schedules(q, 3, &lat) != GBGEMM_OK) return GBGEMM_ERR_CUDA;
+  float direct_us = -1.f;
+  if (h->tuner.measure_schedules(q, 3, &lat, &direct_us) != GBGEMM_OK) return GBGEMM_ERR_CUDA;
   for (int s = 0; s < GBGEMM_NUM_SCHEDULES; ++s) {
     if (lat[(size_t)s] < 0.f || !schedule_allowed(h, q, s)) continue;
     if (*best < 0 || lat[(size_t)s] < lat[(size_t)*best]) *best = s;
   }
+  *direct = direct_us >= 0.f && (*best < 0 || direct_us < lat[(size_t)*best]);
   return GBGEMM_OK;
 }
 
@@ -326,20 +335,42 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
     return GBGEMM_OK;
   }
   gbg::Problem p{ta, tb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
-  gbg::Schedule d = default_schedule(h, h->path, m, n, k, batch);
-  bool fixed = true;  // the fixed heuristic chose
+  const gbg::Schedule fixed = default_schedule(h, h->path, m, n, k, batch);
+  gbg::Schedule d = fixed;
+  bool direct = true;  // a call without a packing pass may serve it (path AUTO)
   const gbgemm_problem q1{transa, transb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
   if (batch == 1 && h->pinned_schedule >= 0 && schedule_allowed(h, q1, h->pinned_schedule)) {
     gbg::schedule_resolve(h->pinned_schedule, m, n, k, alpha, h->num_sms, &d);
-    fixed = false;
+    direct = false;
   } else if (h->tuning >= 1 && batch == 1) {
     const gbgemm_problem q{transa, transb, m, n, k, alpha, beta, A, lda, B, ldb, C, ldc};
     int best = -1;
-    const int rc = choose_schedule(h, q, &best);
+    const int rc = choose_schedule(h, q, &best, &direct);
     if (rc != GBGEMM_OK) return rc;
     if (best >= 0) gbg::schedule_resolve(best, m, n, k, alpha, h->num_sms, &d);
-    fixed = best < 0;
+    else direct = true;
   }
+  gbg::SplitCall c;
+  c.ta = ta; c.tb = tb; c.m = m; c.n = n; c.k = k; c.alpha = alpha; c.beta = beta;
+  c.A = A; c.lda = lda; c.B = B; c.ldb = ldb; c.C = C; c.ldc = ldc;
+  c.batch = batch; c.sa = sa; c.sb = sb; c.sc = sc;
+  c.status = h->d_status; c.num_sms = h->num_sms;
+  gbg::DirectPlan plan;
+  if (direct && h->path == GBGEMM_PATH_AUTO && fixed.path == GBGEMM_PATH_SPLIT_BF16 &&
+      gbg::direct_plan(c, h->num_sms, &plan)) {
+    const int rc = ensure_workspace(h, gbg::direct_workspace_bytes(m, n, plan));
+    if (rc != GBGEMM_OK) return rc;
+    c.ws = h->ws;
+    if (prof_pair(h, &c.gemm_begin, &c.gemm_end) != cudaSuccess) return GBGEMM_ERR_CUDA;
+    if (gbg::launch_direct(c, plan, h->stream) != cudaSuccess) return GBGEMM_ERR_CUDA;
+    h->kernel_launches += plan.slices > 1 && !plan.in_cluster ? 2 : 1;
+    h->gemm_launches += 1;
+    h->last_path = GBGEMM_PATH_SPLIT_BF16;
+    h->last_schedule = gbg::schedule_encode_split(fixed.bn, fixed.raster, batch == 1 ? fixed.level : 0);
+    h->last_direct = 1;
+    return GBGEMM_OK;
+  }
+  h->last_direct = 0;
   const int path = d.path;
   const int simt_cfg = d.simt_cfg, split_bn = d.bn;
   if (path == GBGEMM_PATH_SIMT) {
@@ -351,24 +382,6 @@ static int run_sgemm(gbgemm_handle* h, int ta, int tb, char transa, char transb,
     return GBGEMM_OK;
   }
   if (!split_supported(h)) return GBGEMM_ERR_UNSUPPORTED_DEVICE;
-  gbg::SplitCall c;
-  c.ta = ta; c.tb = tb; c.m = m; c.n = n; c.k = k; c.alpha = alpha; c.beta = beta;
-  c.A = A; c.lda = lda; c.B = B; c.ldb = ldb; c.C = C; c.ldc = ldc;
-  c.batch = batch; c.sa = sa; c.sb = sb; c.sc = sc;
-  c.status = h->d_status; c.num_sms = h->num_sms;
-  gbg::DirectPlan plan;
-  if (fixed && h->path == GBGEMM_PATH_AUTO && gbg::direct_plan(c, h->num_sms, &plan)) {
-    const int rc = ensure_workspace(h, gbg::direct_workspace_bytes(m, n, plan));
-    if (rc != GBGEMM_OK) return rc;
-    c.ws = h->ws;
-    if (prof_pair(h, &c.gemm_begin, &c.gemm_end) != cudaSuccess) return GBGEMM_ERR_CUDA;
-    if (gbg::launch_direct(c, plan, h->stream) != cudaSuccess) return GBGEMM_ERR_CUDA;
-    h->kernel_launches += plan.slices > 1 && !plan.in_cluster ? 2 : 1;
-    h->gemm_launches += 1;
-    h->last_path = GBGEMM_PATH_SPLIT_BF16;
-    h->last_schedule = gbg::schedule_encode_split(split_bn, d.raster, batch == 1 ? d.level : 0);
-    return GBGEMM_OK;
-  }
   // Workspace (one problem or a strided batch): control words, band counters
   // and row maxima (zeroed per call), the packed panels, and with split-K
   // (one problem, long k, too few tiles for the SMs) splitk x tiles raw
@@ -1106,6 +1119,13 @@ int gbgemm_last_schedule(gbgemm_handle* h, int* s) {
   if (!h) return GBGEMM_ERR_NOT_INITIALIZED;
   if (!s) return GBGEMM_ERR_INVALID_VALUE;
   *s = h->last_schedule;
+  return GBGEMM_OK;
+}
+
+int gbgemm_last_direct(gbgemm_handle* h, int* direct) {
+  if (!h) return GBGEMM_ERR_NOT_INITIALIZED;
+  if (!direct) return GBGEMM_ERR_INVALID_VALUE;
+  *direct = h->last_direct;
   return GBGEMM_OK;
 }
 

@@ -138,11 +138,12 @@ int Tuner::time_us(const std::function<cudaError_t()>& run, int reps, float* us)
   return GBGEMM_OK;
 }
 
-int Tuner::measure_schedules(const gbgemm_problem& q0, int reps, std::vector<float>* out) {
+int Tuner::measure_schedules(const gbgemm_problem& q0, int reps, std::vector<float>* out, float* direct) {
   const std::string key = tune_key(q0);
   auto it = sched_cache.find(key);
   if (it != sched_cache.end()) {
-    *out = it->second;
+    out->assign(it->second.begin(), it->second.begin() + GBGEMM_NUM_SCHEDULES);
+    if (direct) *direct = it->second[GBGEMM_NUM_SCHEDULES];
     return GBGEMM_OK;
   }
   const int ta = (q0.transa == 'N' || q0.transa == 'n') ? 0 : 1;
@@ -153,29 +154,40 @@ int Tuner::measure_schedules(const gbgemm_problem& q0, int reps, std::vector<flo
     if (schedule_resolve(sc, q0.m, q0.n, q0.k, q0.alpha, num_sms_, &d) && d.path == GBGEMM_PATH_SPLIT_BF16)
       ws = std::max(ws, split_layout(q0.m, q0.n, q0.k, 1, d.splitk, d.bn).total);
   }
+  if (ws > 0) ws = std::max(ws, split_layout(q0.m, q0.n, q0.k, 1, 1, 256).total);  // covers a direct call's
   gbgemm_problem q;
   uint8_t* wsp = nullptr;
   int rc = scratch(q0, ws, &q, &wsp);
   if (rc != GBGEMM_OK) return rc;
   Problem p{ta, tb, q.m, q.n, q.k, 1.0f, 0.0f, q.A, q.lda, q.B, q.ldb, q.C, q.ldc};
-  std::vector<float> lat((size_t)GBGEMM_NUM_SCHEDULES, -1.f);
+  std::vector<float> lat((size_t)GBGEMM_NUM_SCHEDULES + 1, -1.f);
+  auto call = [&]() {
+    SplitCall c;
+    c.ta = ta; c.tb = tb; c.m = q.m; c.n = q.n; c.k = q.k; c.alpha = 1.0f; c.beta = 0.0f;
+    c.A = q.A; c.lda = q.lda; c.B = q.B; c.ldb = q.ldb; c.C = q.C; c.ldc = q.ldc;
+    c.ws = wsp; c.status = status_; c.num_sms = num_sms_;
+    return c;
+  };
   for (int sc = 0; sc < GBGEMM_NUM_SCHEDULES; ++sc) {
     Schedule d;
     if (!schedule_resolve(sc, q.m, q.n, q.k, q.alpha, num_sms_, &d)) continue;
     auto run = [&]() -> cudaError_t {
       if (d.path == GBGEMM_PATH_SIMT) return launch_simt(p, d.simt_cfg, stream_);
-      SplitCall c;
-      c.ta = ta; c.tb = tb; c.m = q.m; c.n = q.n; c.k = q.k; c.alpha = 1.0f; c.beta = 0.0f;
-      c.A = q.A; c.lda = q.lda; c.B = q.B; c.ldb = q.ldb; c.C = q.C; c.ldc = q.ldc;
+      SplitCall c = call();
       c.bn = d.bn; c.raster = d.raster; c.splitk = d.splitk;
-      c.ws = wsp; c.status = status_; c.num_sms = num_sms_;
       return launch_split_call(c, stream_);
     };
     rc = time_us(run, reps, &lat[(size_t)sc]);
     if (rc != GBGEMM_OK) return rc;
   }
+  DirectPlan plan;
+  if (q.k >= kSplitMinK && ws > 0 && direct_plan(call(), num_sms_, &plan)) {
+    rc = time_us([&] { return launch_direct(call(), plan, stream_); }, reps, &lat[GBGEMM_NUM_SCHEDULES]);
+    if (rc != GBGEMM_OK) return rc;
+  }
   sched_cache[key] = lat;
-  *out = lat;
+  out->assign(lat.begin(), lat.begin() + GBGEMM_NUM_SCHEDULES);
+  if (direct) *direct = lat[GBGEMM_NUM_SCHEDULES];
   return GBGEMM_OK;
 }
 
@@ -274,7 +286,8 @@ int Tuner::save(const char* path) const {
     for (int c = 0; c < GBGEMM_NUM_CONFIGS; ++c) std::fprintf(f, " %.4f", kv.second.cost_us[c]);
     std::fprintf(f, "\n");
   }
-  // schedule latencies: "S key | latency_us x GBGEMM_NUM_SCHEDULES"
+  // schedule latencies: "S key | latency_us x GBGEMM_NUM_SCHEDULES", then that of
+  // the call without a packing pass (a file without it leaves it out of the choice)
   for (const auto& kv : sched_cache) {
     std::fprintf(f, "S %s |", kv.first.c_str());
     for (float v : kv.second) std::fprintf(f, " %.4f", v);
@@ -296,7 +309,7 @@ int Tuner::load(const char* path) {
       if (!bar) { rc = GBGEMM_ERR_INVALID_VALUE; break; }
       std::string key(line + 2, bar - line - 2);
       while (!key.empty() && key.back() == ' ') key.pop_back();
-      std::vector<float> lat((size_t)GBGEMM_NUM_SCHEDULES);
+      std::vector<float> lat((size_t)GBGEMM_NUM_SCHEDULES + 1, -1.f);
       bool ok = true;
       char* sp = bar + 1;
       for (int c = 0; c < GBGEMM_NUM_SCHEDULES && ok; ++c) {
@@ -306,6 +319,9 @@ int Tuner::load(const char* path) {
         sp = end;
       }
       if (!ok) { rc = GBGEMM_ERR_INVALID_VALUE; break; }
+      char* end = nullptr;
+      const float direct = std::strtof(sp, &end);
+      if (end != sp) lat[GBGEMM_NUM_SCHEDULES] = direct;
       sched_cache[key] = lat;
       continue;
     }

@@ -27,12 +27,14 @@ class Tuner {
   // Time every legal configuration of q's shape (cached).  Synchronises the stream.
   int measure(const gbgemm_problem& q, int reps, TuneResult* out);
   // Latency of every legal single-call schedule of q's shape (GBGEMM_NUM_SCHEDULES
-  // entries, -1 illegal; cached).  Synchronises the stream.
-  int measure_schedules(const gbgemm_problem& q, int reps, std::vector<float>* out);
+  // entries, -1 illegal; cached), and in *direct (may be null) that of the call
+  // without a packing pass that path AUTO would make (-1 where it makes none,
+  // or a loaded file does not say).  Synchronises the stream.
+  int measure_schedules(const gbgemm_problem& q, int reps, std::vector<float>* out, float* direct = nullptr);
   int save(const char* path) const;
   int load(const char* path);
   std::map<std::string, TuneResult> cache;
-  std::map<std::string, std::vector<float>> sched_cache;
+  std::map<std::string, std::vector<float>> sched_cache;  // GBGEMM_NUM_SCHEDULES latencies, then the direct call's
 
  private:
   int ensure(size_t bytes);

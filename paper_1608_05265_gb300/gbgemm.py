@@ -72,7 +72,7 @@ EXPORTS = [
     "gbgemm_predictor_get", "gbgemm_predictor_features", "gbgemm_predictor_predict",
     "gbgemm_predictor_loss_grad", "gbgemm_predictor_train", "gbgemm_check_error",
     "gbgemm_schedule_info", "gbgemm_schedule_legal", "gbgemm_schedule_default", "gbgemm_autotune_schedules",
-    "gbgemm_last_schedule", "gbgemm_set_schedule", "gbgemm_predictor_select",
+    "gbgemm_last_schedule", "gbgemm_last_direct", "gbgemm_set_schedule", "gbgemm_predictor_select",
 ]
 
 _lock = threading.Lock()
@@ -151,6 +151,7 @@ def lib():
             L.gbgemm_schedule_default.argtypes = [vp, PP, ip]
             L.gbgemm_autotune_schedules.argtypes = [vp, PP, ctypes.c_int, fp, ip]
             L.gbgemm_last_schedule.argtypes = [vp, ip]
+            L.gbgemm_last_direct.argtypes = [vp, ip]
             L.gbgemm_set_schedule.argtypes = [vp, ctypes.c_int]
             L.gbgemm_predictor_select.argtypes = [vp, ctypes.c_int]
             L.gbgemm_profile_begin.argtypes = [vp]
@@ -169,8 +170,8 @@ def lib():
                          "gbgemm_predictor_get", "gbgemm_predictor_features", "gbgemm_predictor_predict",
                          "gbgemm_predictor_loss_grad", "gbgemm_predictor_train", "gbgemm_check_error",
                          "gbgemm_schedule_info", "gbgemm_schedule_legal", "gbgemm_schedule_default",
-                         "gbgemm_autotune_schedules", "gbgemm_last_schedule", "gbgemm_set_schedule",
-                         "gbgemm_predictor_select"):
+                         "gbgemm_autotune_schedules", "gbgemm_last_schedule", "gbgemm_last_direct",
+                         "gbgemm_set_schedule", "gbgemm_predictor_select"):
                 getattr(L, name).restype = ctypes.c_int
             _lib = L
     return _lib
@@ -385,6 +386,12 @@ class Handle:
         v = ctypes.c_int()
         _check("gbgemm_last_schedule", lib().gbgemm_last_schedule(self._h, ctypes.byref(v)))
         return v.value
+
+    def last_direct(self) -> bool:
+        """Whether that call ran without a packing pass, which no schedule describes."""
+        v = ctypes.c_int()
+        _check("gbgemm_last_direct", lib().gbgemm_last_direct(self._h, ctypes.byref(v)))
+        return bool(v.value)
 
     def predictor_predict(self, x, legal, scores=None, configs=None):
         """Device tensors: x (n x 8 float32), legal (n uint8); fills scores (n x 6) and configs (n int32)."""
