@@ -3,7 +3,7 @@
 // tiles of one problem (or a strided batch) in a rasterised order,
 // GroupedSched walks the tiles of many problems, problem after problem.  The
 // per-tile job carries everything a role needs, including the tile width BN
-// (64, 128 or 256) as a run-time value: the MMA instruction descriptor, the
+// (64, 128 or 256; pairs: any multiple of 32 up to 256) as a run-time value: the MMA instruction descriptor, the
 // B copy size and the epilogue width all follow it, and shared memory and
 // TMEM are sized for MAXBN.
 //
@@ -38,9 +38,9 @@
 //   warp 18         with beta != 0 and k <= 512, asks L2 for each tile's C
 //                   columns as soon as the tile is handed out, so that the
 //                   epilogue's reads of C find them there;
-//   warp 19         with staged jobs (many problems) draws the tiles and
-//                   leaves each tile's job in shared memory, ahead of the
-//                   producer (else idle).
+//   warp 19         only with staged jobs (many problems): draws the tiles
+//                   and leaves each tile's job in shared memory, ahead of the
+//                   producer.
 //
 // What bounds the many-problem instance is the two single-thread roles: at
 // 4096 problems up to 1024^3 the issuer spent about 80 cycles per MMA and the
@@ -114,9 +114,10 @@ struct alignas(16) TileJob {
   size_t a_kstride;         // bytes between k chunks of the A panel
   size_t b_kstride;         // bytes between k chunks of the B panel
   int nkc;                  // k chunks
-  int bn;                   // tile width: 64, 128 or 256
+  int bn;                   // tile width: 64, 128 or 256; of a pair, a multiple of 32 in 32 .. 256
   int parts;                // 1: [hi | lo] panels, 3 products; 2: also compact lo3 panels, 6 products
-  int a_rows, b_rows;       // A and B panel rows copied per k chunk (b_rows: also the MMA's N; pairs: whole blocks)
+  int a_rows, b_rows;       // A and B panel rows copied per k chunk.  b_rows is also the MMA's N: at most bn, a
+                            // multiple of 16; of a pair, of 32, half of it from a multiple of 16 rows on in each CTA
   int group;                // staged jobs: k chunks per ring slot (what fits beside each other), else 1
   int64_t a_part, b_part;   // byte offsets from the [hi | mid] panels to the compact lo3 panels
   int64_t m0, n0;           // tile origin in C
@@ -481,11 +482,12 @@ __global__ void __launch_bounds__(256, 4) pack_tasks_kernel(const Sched S) {
 // One CTA per SM.  Registers are handed out to whole groups of four warps,
 // so the 19 warps are charged as 20: 96 registers per thread.
 //
-// PAIR: launched in clusters of two CTAs on two SMs, each pair computing
-// 256 x 256 tiles (SingleSched pair items) with tcgen05 MMAs of
-// cta_group::2.  Each CTA loads its own 128-row A block and half of the
-// tile's 256 B rows, so per SM a k chunk brings 32 KiB instead of 48 KiB and
-// the tensor cores read half as many B bytes from shared memory.  The even
+// PAIR: launched in clusters of two CTAs on two SMs, each pair computing tiles
+// of 256 rows and up to 256 columns (a multiple of 32; SingleSched pair items,
+// choose_pair_tiles) with tcgen05 MMAs of cta_group::2.  Each CTA loads its
+// own 128-row A block and half of the tile's B rows, so per SM a k chunk of
+// the widest tile brings 32 KiB instead of 48 KiB and the tensor cores read
+// half as many B bytes from shared memory.  The even
 // CTA (rank 0) issues the MMAs for both; the odd CTA's warp 1 relays each
 // of its landed stages to rank 0's "full" barrier (which then counts two
 // arrivals), its epilogue warps release the accumulator on rank 0's

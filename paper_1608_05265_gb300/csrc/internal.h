@@ -105,6 +105,9 @@ struct PairTiles {
   double us = 0.0;  // estimated time of the launch
 };
 PairTiles choose_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks, bool three, int pairs);
+// The rule alone, for tests (no GPU): tiles[0 .. 2] = bn, tiles, tail_start.
+extern "C" void gbgemm_internal_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks, int three, int pairs,
+                                           int64_t* tiles);
 
 // Workspace of one split-path call (or strided batch), in bytes from its
 // start: [control words | band counters | row maxima | per problem: panel A,

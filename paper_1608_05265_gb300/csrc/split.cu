@@ -68,8 +68,8 @@ __device__ __forceinline__ void rescale_slices(float4& acc, const float4* p, siz
 // vectors), the slices' raw accumulators summed in slice order
 // (deterministic), then the epilogue of split_gemm_kernel: x 2^(e_i + f_j),
 // alpha, and beta C with one rounding of beta C and one fused multiply-add.
-// With pexp the slices have exponents of their own (direct.cu).  Every load of a thread is independent, so one pass over the grid keeps
-// them all in flight.
+// With pexp the slices have exponents of their own (direct.cu).  Every load of
+// a thread is independent, so one pass over the grid keeps them all in flight.
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n, int bn, int tiles_m, int tiles_n,
                                                             int splitk, const float* __restrict__ partial,
                                                             const uint32_t* __restrict__ amaxA,
@@ -265,6 +265,12 @@ PairTiles choose_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks,
   return best;
 }
 
+extern "C" void gbgemm_internal_pair_tiles(int64_t m, int64_t n, int64_t batch, int64_t chunks, int three, int pairs,
+                                           int64_t* tiles) {
+  const PairTiles t = choose_pair_tiles(m, n, batch, chunks, three != 0, pairs);
+  tiles[0] = t.bn; tiles[1] = t.tiles; tiles[2] = t.tail_start;
+}
+
 namespace {
 
 // The head of the workspace (control words, band counters, row maxima) set to
@@ -352,6 +358,9 @@ cudaError_t launch_split_call(const SplitCall& c, cudaStream_t s) {
     S.tail_start = (int)pair_items;
     if (splitk == 1) {
       const PairTiles T = choose_pair_tiles(c.m, c.n, c.batch, nkc, S.parts == 2, pair_cap);
+      // what job_pair and the epilogue's column split rest on
+      const int narrow = T.tail_start < T.tiles ? T.bn / 2 : T.bn;
+      if (T.bn < 64 || T.bn > kMaxBN || narrow % 32 != 0) return cudaErrorInvalidValue;
       if (2 * T.tiles <= (int64_t)0x7FFFFFFF) {
         S.bn = T.bn;
         S.tiles_n = (int)((c.n + T.bn - 1) / T.bn);
