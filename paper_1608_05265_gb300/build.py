@@ -43,8 +43,8 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(CSRC, v[1]) for v in VARIANTS] + [h for h in HEADERS if os.path.exists(h)] + \
-        [os.path.abspath(__file__)]
+    deps = [os.path.join(CSRC, s) for s in SOURCES + [v[1] for v in VARIANTS]] + \
+        [h for h in HEADERS if os.path.exists(h)] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

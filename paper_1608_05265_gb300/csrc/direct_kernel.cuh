@@ -400,7 +400,8 @@ __device__ __forceinline__ void tmem_sum16(uint32_t taddr, float (&v)[16]) {
 }
 
 template <int BN, bool PAIR, int PARTS, int MA, int MB>
-__global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectShape<BN, PAIR, PARTS>::CTAS) direct_gemm_kernel(const DirectArgs S) {
+__global__ void __launch_bounds__(DirectShape<BN, PAIR, PARTS>::THREADS, DirectShape<BN, PAIR, PARTS>::CTAS)
+    direct_gemm_kernel(const DirectArgs S) {
   using D = DirectShape<BN, PAIR, PARTS>;
   constexpr int BS = D::BS, UK = D::UK;
   // With two parts, steps with K-vectors to watch have a loop of their own: its

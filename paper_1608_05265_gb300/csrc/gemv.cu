@@ -89,7 +89,8 @@ __global__ void __launch_bounds__(kGemvNThreads, 2) gemv_n_kernel(int64_t m, int
       } else if (VEC && rows == 4) {  // the last columns
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const float4 f = u < cnt ? __ldg(reinterpret_cast<const float4*>(col + u * lda)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 f = u < cnt ? __ldg(reinterpret_cast<const float4*>(col + u * lda)) : zero;
           w[u][0] = f.x; w[u][1] = f.y; w[u][2] = f.z; w[u][3] = f.w;
         }
       } else {  // the last columns, or the last rows
@@ -301,7 +302,9 @@ cudaError_t launch_gemv(bool trans, int64_t m, int64_t n, float alpha, const flo
     const int rt = m <= 256 ? 64 : m <= 1024 ? 128 : vec ? (slice <= 64 ? 128 : 256) : 64;
     const dim3 grid((unsigned)ceil_div(m, 4 * rt), (unsigned)ceil_div(n, slice));
     if (ceil_div(m, 4 * rt) > 0x7FFFFFFF) return cudaErrorInvalidConfiguration;
-    auto kernel = vec ? (rt == 64 ? gemv_n_kernel<true, 64> : rt == 128 ? gemv_n_kernel<true, 128> : gemv_n_kernel<true, 256>)
+    auto kernel = vec ? (rt == 64    ? gemv_n_kernel<true, 64>
+                         : rt == 128 ? gemv_n_kernel<true, 128>
+                                     : gemv_n_kernel<true, 256>)
                       : (rt == 64 ? gemv_n_kernel<false, 64> : gemv_n_kernel<false, 128>);
     kernel<<<grid, kGemvNThreads, 0, s>>>(m, n, A, lda, x, incx, slice, part, alpha, beta, y, incy);
     slices = grid.y;

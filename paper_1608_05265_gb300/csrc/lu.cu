@@ -1137,13 +1137,14 @@ __device__ __forceinline__ float quotient(float x, float d, float r) {
 
 // Solve the staged triangle in place on ys (w values), in steps of 32 rows.
 // Warp 0 solves a step's 32 x 32 triangle and carries its contribution to the
-// next 32 rows along (the same shuffled values, off the chain); the other threads meanwhile apply the step before to the rows after
-// those, so a step is one barrier and the chain of shuffles and multiply-adds.
+// next 32 rows along (the same shuffled values, off the chain); the other
+// threads meanwhile apply the step before to the rows after those, so a step
+// is one barrier and the chain of shuffles and multiply-adds.
 // The back substitution's division is a reciprocal, taken ahead, and four
 // multiply-adds on the chain; a step that meets a value outside their range
 // (a zero, a tiny or huge one, infinity, NaN) runs again with divisions.  The
-// loops stay rolled: unrolled 32 times they waited for instructions.  Every thread of the block calls it (it
-// synchronises); at least 256 threads.
+// loops stay rolled: unrolled 32 times they waited for instructions.  Every
+// thread of the block calls it (it synchronises); at least 256 threads.
 // Measured at n = 4608 (18 blocks of 256 rows, one right-hand side): forward
 // sweep 235 -> 201 us, back 419 -> 227 us; what bounds both is the chain, about
 // 45 cycles a row, and the hand-over of a block's solution.
@@ -1400,7 +1401,8 @@ cudaError_t launch_panel_reg(int C, int T, int n, float* A, int64_t lda, int j0,
   auto bytes = [](int blocks, int threads) {
     return (size_t)kLuPanelNb * (RPT * threads + blocks * kLuPanelNb) * sizeof(float);
   };
-  cudaError_t e = set_smem_once(fn, 6 + 2 * RPT + CLUSTER, std::max(bytes(CLUSTER ? kLuPanelCluster : 1, kRegPanelThreads), kRegPanelAlone));
+  cudaError_t e = set_smem_once(fn, 6 + 2 * RPT + CLUSTER,
+                                std::max(bytes(CLUSTER ? kLuPanelCluster : 1, kRegPanelThreads), kRegPanelAlone));
   if (e != cudaSuccess) return e;
   static bool wide_set[64] = {};
   int dev = 0;
@@ -1449,10 +1451,9 @@ cudaError_t launch_lu_panel(int n, float* A, int64_t lda, int j0, int nbp, int* 
                                 : rpt == 2 ? launch_panel_reg<2, true>
                                 : rpt == 3 ? launch_panel_reg<3, true>
                                            : launch_panel_reg<4, true>)
-                             : (rpt == 1   ? launch_panel_reg<1, false>
+                             : (rpt == 1   ? launch_panel_reg<1, false>  // (at most 384 rows)
                                 : rpt == 2 ? launch_panel_reg<2, false>
-                                : rpt == 3 ? launch_panel_reg<3, false>
-                                           : launch_panel_reg<4, false>);
+                                           : launch_panel_reg<3, false>);
     cudaError_t e = launch(blocks, T, n, A, lda, j0, nbp, ipiv, info, perm, status, s, jp, nbq, perm_prev);
     if (e == cudaSuccess || C != kLuPanelCluster) return e;
     cudaGetLastError();
