@@ -38,16 +38,19 @@ namespace {
 // slice's tile has exponents: every slice's are first brought to the largest
 // exponent of the row and of the column (a slice where either is zero
 // throughout has kNoExp there and adds nothing).
-__device__ __noinline__ float4 rescaled_sum(const float4* p, size_t slice_elems, int splitk, const int* pexp,
-                                            size_t pstride, int row, int col) {
+__device__ __forceinline__ float4 rescaled_sum(const float4* p, size_t slice_elems, int splitk, const int* pexp,
+                                               size_t pstride, int row, int col) {
   float out[4];
+#pragma unroll 1
   for (int q = 0; q < 4; ++q) {
     int er = kNoExp, ec = kNoExp;
+#pragma unroll 1
     for (int s = 0; s < splitk; ++s) {
       er = max(er, pexp[s * pstride + 1 + row + q]);
       ec = max(ec, pexp[s * pstride + 129 + col]);
     }
     float sum = 0.f;
+#pragma unroll 1
     for (int s = 0; s < splitk; ++s) {
       const float acc = reinterpret_cast<const float*>(p + s * (slice_elems / 4))[q];
       sum += scale_up(acc, pexp[s * pstride + 1 + row + q] - er + pexp[s * pstride + 129 + col] - ec);
@@ -68,14 +71,19 @@ __device__ __forceinline__ void rescale_slices(float4& acc, const float4* p, siz
 // vectors), the slices' raw accumulators summed in slice order
 // (deterministic), then the epilogue of split_gemm_kernel: x 2^(e_i + f_j),
 // alpha, and beta C with one rounding of beta C and one fused multiply-add.
-// With pexp the slices have exponents of their own (direct.cu).  Every load of
-// a thread is independent, so one pass over the grid keeps them all in flight.
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n, int bn, int tiles_m, int tiles_n,
-                                                            int splitk, const float* __restrict__ partial,
-                                                            const uint32_t* __restrict__ amaxA,
-                                                            const uint32_t* __restrict__ amaxB,
-                                                            const int* __restrict__ pexp, float alpha, float beta,
-                                                            float* __restrict__ C, int64_t ldc) {
+// EXP: the slices have exponents of their own (pexp, direct.cu) instead of the
+// operands' maxima.  Every load of a thread is independent, so one pass over
+// the grid keeps them all in flight: the kernel is as fast as its blocks are
+// many on an SM (1024^2 outputs of 4 slices, cold: 8.3 us; 13.2 with 128
+// registers).  U slices' loads are in flight: eight, or sixteen where a small
+// output gives no SM more than two blocks (300 x 300 x 5000, 31 slices: a call
+// 33.2 -> 32.1 us).
+template <bool EXP, int U>
+__global__ void __launch_bounds__(256, U == 8 ? 4 : 2)
+    splitk_reduce_kernel(int64_t m, int64_t n, int bn, int tiles_m, int tiles_n, int splitk,
+                         const float* __restrict__ partial, const uint32_t* __restrict__ amaxA,
+                         const uint32_t* __restrict__ amaxB, const int* __restrict__ pexp, float alpha, float beta,
+                         float* __restrict__ C, int64_t ldc) {
   wait_prerequisite_grid();  // launched as a dependent of the GEMM
   const int64_t mq = (m + 3) / 4, total = mq * n;
   const size_t tile_elems = (size_t)128 * bn, slice_elems = (size_t)tiles_m * tiles_n * tile_elems;
@@ -86,19 +94,19 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
     const float4* p = reinterpret_cast<const float4*>(
         partial + (size_t)(tm * tiles_n + tn) * tile_elems + (size_t)(j - tn * bn) * 128 + (i0 & 127));
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < splitk; s0 += 8) {
-      // eight slices' loads in flight, then summed in slice order
-      float4 v[8];
+    for (int s0 = 0; s0 < splitk; s0 += U) {
+      // U slices' loads in flight, then summed in slice order
+      float4 v[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < U; ++u)
         if (s0 + u < splitk) v[u] = __ldcs(p + (size_t)(s0 + u) * (slice_elems / 4));
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < U; ++u)
         if (s0 + u < splitk) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
     }
-    if (pexp) rescale_slices(acc, p, slice_elems, splitk, pexp + (tm * tiles_n + tn) * kDirectExpInts,
-                             (size_t)tiles_m * tiles_n * kDirectExpInts, (int)(i0 & 127), (int)(j - tn * bn));
-    const int fj = amaxB ? scale_exp_from_bits(amaxB[j]) : 0;
+    if (EXP) rescale_slices(acc, p, slice_elems, splitk, pexp + (tm * tiles_n + tn) * kDirectExpInts,
+                            (size_t)tiles_m * tiles_n * kDirectExpInts, (int)(i0 & 127), (int)(j - tn * bn));
+    const int fj = EXP ? 0 : scale_exp_from_bits(amaxB[j]);
     float* c = C + i0 + j * ldc;
     const float a4[4] = {acc.x, acc.y, acc.z, acc.w};
     float o[4];
@@ -107,7 +115,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
       const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int e = amaxA ? scale_exp_from_bits(amaxA[i0 + q]) + fj : 0;
+        const int e = EXP ? 0 : scale_exp_from_bits(amaxA[i0 + q]) + fj;
         const float v = (e >= -126 && e <= 127) ? a4[q] * __int_as_float((e + 127) << 23) : scalbnf(a4[q], e);
         o[q] = (beta != 0.f) ? fmaf(alpha, v, beta * c4[q]) : alpha * v;
       }
@@ -116,7 +124,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(int64_t m, int64_t n
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         if (i0 + q >= m) break;
-        const int e = amaxA ? scale_exp_from_bits(amaxA[i0 + q]) + fj : 0;
+        const int e = EXP ? 0 : scale_exp_from_bits(amaxA[i0 + q]) + fj;
         const float v = (e >= -126 && e <= 127) ? a4[q] * __int_as_float((e + 127) << 23) : scalbnf(a4[q], e);
         c[q] = (beta != 0.f) ? fmaf(alpha, v, beta * c[q]) : alpha * v;
       }
@@ -390,7 +398,7 @@ cudaError_t launch_splitk_reduce(const SplitGemmArgs& a, cudaStream_t s) {
   const int tm = (int)((a.m + 127) / 128), tn = (int)((a.n + a.bn - 1) / a.bn);
   const int64_t total = (a.m + 3) / 4 * a.n;  // a thread per four rows of a column
   int64_t blocks = (total + 255) / 256;
-  const int64_t cap = (int64_t)(a.num_sms > 0 ? a.num_sms : 148) * 16;
+  const int64_t sms = a.num_sms > 0 ? a.num_sms : 148, cap = sms * 16;
   if (blocks > cap) blocks = cap;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks);
@@ -401,7 +409,10 @@ cudaError_t launch_splitk_reduce(const SplitGemmArgs& a, cudaStream_t s) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, splitk_reduce_kernel, a.m, a.n, a.bn, tm, tn, a.splitk, (const float*)a.partial,
+  const bool deep = a.splitk > 8 && blocks <= 2 * sms;
+  auto* kernel = a.partial_exp ? (deep ? splitk_reduce_kernel<true, 16> : splitk_reduce_kernel<true, 8>)
+                               : (deep ? splitk_reduce_kernel<false, 16> : splitk_reduce_kernel<false, 8>);
+  return cudaLaunchKernelEx(&cfg, kernel, a.m, a.n, a.bn, tm, tn, a.splitk, (const float*)a.partial,
                             a.amaxA, a.amaxB, a.partial_exp, a.alpha, a.beta, a.C, a.ldc);
 }
 
