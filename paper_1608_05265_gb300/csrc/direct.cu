@@ -80,7 +80,9 @@ double direct_us(const DirectPlan& p, int64_t m, int64_t n, int64_t k, int64_t b
   const double out = three ? 0.0 : p.bn * 0.018;  // a tile's way out: not hidden behind the next one
   double t = (three ? 6.7 : 5.2) + waves * (steps * step + out) + (waves - 1) * again;
   if (p.slices > 1)
-    t += !p.in_cluster ? 7.0 : three ? 0.9 * ((p.bn / p.slices + 7) / 8) + 0.2 * p.slices : 1.15 * ((p.bn / p.slices + 15) / 16);
+    t += !p.in_cluster ? 7.0
+         : three       ? 0.9 * ((p.bn / p.slices + 7) / 8) + 0.2 * p.slices
+                       : 1.15 * ((p.bn / p.slices + 15) / 16);
   return t;
 }
 
@@ -92,9 +94,9 @@ bool choose_plan(const SplitCall& c, int num_sms, int max_cluster, DirectPlan* p
   const int64_t nkc = panel_k_chunks(k);
   const int scalars = (load_mode(c.ta == 1, c.A, c.lda, batch > 1 ? c.sa : 0) == kScalar) +
                       (load_mode(c.tb == 0, c.B, c.ldb, batch > 1 ? c.sb : 0) == kScalar);
-  // In favour of the packed path, for the estimates' error.  Over 500 further
-  // calls drawn alike, path AUTO then takes 0.745 times the packed path's time
-  // in the geometric mean and at most 1.01 times (with 4% both ways up to 1.09).
+  // In favour of the packed path, for the estimates' error.  Over 1500 further
+  // calls drawn alike, path AUTO then takes 0.738 times the packed path's time
+  // in the geometric mean, four of them more than 1.02 times, the worst 1.07.
   const double packed = packed_us(m, n, k, batch, num_sms, three);
   double best = (three ? 0.9 : 0.94) * packed;
   bool found = false;
