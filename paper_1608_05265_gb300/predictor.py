@@ -153,10 +153,14 @@ def default_choice(shapes) -> np.ndarray:
     """The library's fixed heuristic (GBGEMM_CONFIG_DEFAULT) for each shape."""
     out = []
     for (ta, tb, m, n, k, *_rest) in shapes:
-        if k >= 16:
-            out.append(gbgemm.CFG_SPLIT_BN64 if n <= 64 else gbgemm.CFG_SPLIT_BN128)
-        else:
-            out.append(gbgemm.CFG_SIMT_128x128)
+        if k >= 16:  # the widest tile that n fills
+            out.append(gbgemm.CFG_SPLIT_BN64 if n <= 64 else gbgemm.CFG_SPLIT_BN128 if n <= 128
+                       else gbgemm.CFG_SPLIT_BN256)
+        else:  # the least padded area, ties to the larger tile
+            area = lambda bm, bn: -(-m // bm) * bm * (-(-n // bn) * bn)
+            big, wide, small = area(128, 128), area(128, 64), area(64, 64)
+            out.append(gbgemm.CFG_SIMT_128x128 if big <= wide and big <= small
+                       else gbgemm.CFG_SIMT_128x64 if wide <= small else gbgemm.CFG_SIMT_64x64)
     return np.array(out, dtype=np.int64)
 
 
