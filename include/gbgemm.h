@@ -345,7 +345,10 @@ typedef enum {
 typedef struct gbgemm_grouped_plan gbgemm_grouped_plan;
 
 /* probs: host array of `count` problems (device matrix pointers).
- * config_source: a gbgemm_config_source.  On success *plan owns the plan. */
+ * config_source: a gbgemm_config_source.  On success *plan owns the plan.
+ * Device memory (gbgemm_grouped_plan_stats): the problems' split panels, and
+ * beside them 160 bytes per output tile of at most 128 x 256 on the split path
+ * (0.12% of the C of a full one). */
 int gbgemm_grouped_plan_create(gbgemm_handle* h, const gbgemm_problem* probs, int64_t count, int config_source,
                                gbgemm_grouped_plan** plan, int64_t* bad_index);
 /* As gbgemm_grouped_plan_create with the configuration of every problem
