@@ -113,8 +113,8 @@ int default_config(const gbgemm_problem& q) {
   // Edge tiles cost what they hold, so the widest tile that n fills.  A plan
   // with 256 columns from n = 129 on against never: 2200 problems up to 1024
   // 884 against 997 us, 4096 up to 256 332 against 341, 128 up to 1024 86
-  // against 94, 128 up to 256 (fewer tiles than SMs) 28 against 27; from 193 or
-  // 257 on took 2 and 4% longer than from 129 on 4096 problems up to 1024.
+  // against 94; from 193 or 257 on took 2 and 4% longer than from 129 on 4096
+  // problems up to 1024.  (A plan of fewer tiles than SMs: choose_configs.)
   if (q.k >= kSplitShortK && q.alpha != 0.0f)
     return q.n <= 64 ? GBGEMM_CFG_SPLIT_BN64 : q.n <= 128 ? GBGEMM_CFG_SPLIT_BN128 : GBGEMM_CFG_SPLIT_BN256;
   // SIMT: the tile shape with the least padded area (ties to the larger tile)

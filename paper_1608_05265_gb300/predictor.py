@@ -150,7 +150,7 @@ def regret(cost: np.ndarray, choice: np.ndarray) -> dict:
 
 
 def default_choice(shapes) -> np.ndarray:
-    """The library's fixed heuristic (GBGEMM_CONFIG_DEFAULT) for each shape."""
+    """The library's fixed heuristic (GBGEMM_CONFIG_DEFAULT) for each shape, in a plan with more tiles than SMs."""
     out = []
     for (ta, tb, m, n, k, *_rest) in shapes:
         if k >= 16:  # the widest tile that n fills
