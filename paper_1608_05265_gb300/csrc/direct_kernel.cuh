@@ -857,15 +857,16 @@ bool direct_kernel_fits(int cluster) {
     if (const signed char k = known[dev][bit].load(std::memory_order_relaxed)) return k > 0;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  int n = 0;
-  bool fits = prepare_direct_launch<BN, PAIR, PARTS, MA, MB>(dev, cluster, cluster, &cfg, attr) == cudaSuccess;
-  if (fits && cluster > 1) {
+  cudaError_t e = prepare_direct_launch<BN, PAIR, PARTS, MA, MB>(dev, cluster, cluster, &cfg, attr);
+  int n = 1;
+  if (e == cudaSuccess && cluster > 1) {
     cfg.attrs = attr + 1;
     cfg.numAttrs = 1;
-    fits = cudaOccupancyMaxActiveClusters(&n, direct_gemm_kernel<BN, PAIR, PARTS, MA, MB>, &cfg) == cudaSuccess && n > 0;
+    e = cudaOccupancyMaxActiveClusters(&n, direct_gemm_kernel<BN, PAIR, PARTS, MA, MB>, &cfg);
   }
-  if (!fits) (void)cudaGetLastError();  // such a cluster is not used: not an error
-  if (keep) known[dev][bit].store(fits ? 1 : -1, std::memory_order_relaxed);
+  if (e != cudaSuccess) (void)cudaGetLastError();  // no answer: not used this time, and not an error
+  const bool fits = e == cudaSuccess && n > 0;
+  if (keep && e == cudaSuccess) known[dev][bit].store(fits ? 1 : -1, std::memory_order_relaxed);
   return fits;
 }
 
