@@ -16,7 +16,7 @@
 // What bounds both is memory: enough bytes have to be in flight (128 a thread,
 // 16-byte loads where every column starts on 16 bytes) in long pieces of a
 // column.  Measured on GB300 at 16384^2 (1.07 GB), back to back: N 179.6 ->
-// 155.7 us (6.9 TB/s), T 186 -> 148 us; with ld + 1, N 175 -> 172, T 186 ->
+// 154 us (7.0 TB/s), T 186 -> 148 us; with ld + 1, N 175 -> 172, T 186 ->
 // 164; a y of 300 from 12000 columns 22.6 -> 10.4 us (the slices' sums spread
 // over eight threads a row, and that kernel launched ahead).
 // Every sum is formed in the same order on every run (no atomics).
